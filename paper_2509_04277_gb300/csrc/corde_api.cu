@@ -132,12 +132,46 @@ struct Bin {
                     // indexes kSelfVariants)
   int grid = 0;     // 1: the cluster variant's blocks form a cooperative grid
   float4* d_gh = nullptr;  // grid bins: the rods' global exchange slots
+  TilePlan tile;           // per > 0: launches without a mailbox run the tile kernel
+  float4* d_tile_gh = nullptr;  // tiles on a cooperative grid: their exchange buffers
 };
+
+// Tile plan of a bin of `count` rods of at most n nodes whose kernel layout has `arith`
+// elements per thread; per = 0 where the block, cluster or grid kernel runs.
+// The tiles repeat their ghosts' work (three times an element's at two elements per lane, 1.6
+// times at four), so they are for handles that leave SMs idle: every rod has one SM and the
+// tiles take from the `spare` others (which a tile plan reduces).  One warp per SM partition is fastest (512 nodes: 2.15 us/step at 4 warps
+// a block, 2.50 at 6, 2.59 at 8).
+// Two elements per lane shorten the chain of a step (512 nodes: 2.15 against 2.88 us/step at
+// four) and win up to seven warps a block over the largest cluster (2048 nodes: 2.73 against
+// 2.98); longer rods take four (5000 nodes: 3.02 on a cluster, 3.62 at two on a grid).
+TilePlan tile_plan(int n, int count, int arith, int* spare) {
+  TilePlan p;
+  p.arith = arith;
+  const int K2 = tile_count(2, n), K4 = tile_count(4, n);
+  p.per = K2 <= 7 * kMaxCluster ? 2 : 4;
+  const int K = p.per == 2 ? K2 : K4;
+  p.blocks = std::min((K + 3) / 4, kMaxCluster);
+  if (K > 8 * p.blocks) {
+    // more tiles than a cluster holds: a cooperative grid, one block per SM
+    p.grid = 1;
+    p.blocks = std::min(K, *spare + 1);
+  }
+  p.warps = p.blocks > 0 ? (K + p.blocks - 1) / p.blocks : 0;
+  const int64_t more = (int64_t)(p.blocks - 1) * count;
+  if (p.blocks < 1 || p.warps > kTileMaxWarps || (p.grid && count > 1) || *spare < 0 || more > *spare) {
+    p.per = 0;
+  } else {
+    *spare -= (int)more;
+  }
+  return p;
+}
 
 }  // namespace
 
 struct corde_rods {
   int device = 0;
+  int sms = 0;
   int n_rods = 0;
   int64_t n_elem = 0;
   std::vector<int> n_nodes, off;
@@ -389,6 +423,7 @@ void free_bins(rod_handle h) {
   for (auto& b : h->bins) {
     cudaFree(b.d_work);
     cudaFree(b.d_gh);
+    cudaFree(b.d_tile_gh);
   }
   h->bins.clear();
 }
@@ -412,6 +447,7 @@ int build_bins(rod_handle h) {
     if (std::find(keys.begin(), keys.end(), k) == keys.end()) keys.push_back(k);
   }
   std::sort(keys.begin(), keys.end());
+  int spare = h->sms - h->n_rods;
   for (const auto& k : keys) {
     std::vector<int> rods;
     for (int r = 0; r < h->n_rods; ++r)
@@ -428,6 +464,13 @@ int build_bins(rod_handle h) {
       const size_t n4 = rods.size() * 2 * (size_t)b.cluster * kHaloSlots * 2;
       CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
       CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
+    }
+    if (b.cluster >= 0) {
+      int nmax = 0;
+      for (int r : rods) nmax = std::max(nmax, h->n_nodes[r]);
+      const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
+      b.tile = tile_plan(nmax, b.count, arith, &spare);
+      if (b.tile.per && b.tile.grid) CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
     }
     h->bins.push_back(b);
   }
@@ -456,7 +499,13 @@ int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const f
   int launches = 0;
   for (const auto& b : bins) {
     a.work = b.d_work;
-    if (b.cluster < 0) {
+    if (b.tile.per && !mb) {
+      a.grid_halo = b.d_tile_gh;
+      cudaError_t e = launch_tile(a, b.count, b.tile, s);
+      if (e != cudaSuccess)
+        return fail(CORDE_ERR_CUDA, std::string("tile step launch (blocks=") + std::to_string(b.tile.blocks) +
+                                        ", warps=" + std::to_string(b.tile.warps) + "): " + cudaGetErrorString(e));
+    } else if (b.cluster < 0) {
       const StepVariant& v = kSelfVariants[b.variant];
       cudaError_t e = v.launch(a, b.count, s);
       if (e != cudaSuccess)
@@ -681,6 +730,7 @@ int rod_create(int n_rods, const RodParams* params, const float* pos, const floa
 
   rod_handle h = new corde_rods();
   h->device = dev;
+  cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
   h->n_rods = n_rods;
   h->n_elem = E;
   h->n_nodes = nn;
@@ -1149,6 +1199,8 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         if (v.capacity() < nmax) continue;
         if (v.capacity() >= 8 * nmax && v.nt > 32) continue;  // mostly idle threads
         std::vector<Bin> one{Bin{(int)vi, (int)rods.size(), d_work}};
+        int spare = h->sms - h->n_rods;
+        one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &spare);
         restore();
         if ((rc = launch_bins(h, one, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
         float best_rep = 1e30f;
@@ -1344,6 +1396,7 @@ int rod_bind(rod_handle h, int outer, int inner, int mode) {
 // variant, so that rod_rollout and the adjoint's recomputation run the same kernel code.
 static int build_adjoint_bins(rod_handle h) {
   if (!h->adj_bins.empty()) return CORDE_OK;
+  int spare = h->sms - h->n_rods;
   for (int nt = 32; nt <= kAdjointMaxNodes / 2; nt *= 2) {
     std::vector<int> rods;
     for (int r = 0; r < h->n_rods; ++r) {
@@ -1357,6 +1410,7 @@ static int build_adjoint_bins(rod_handle h) {
     Bin b{v, (int)rods.size(), nullptr};
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
+    b.tile = tile_plan(2 * nt, b.count, 2, &spare);
     h->adj_bins.push_back(b);
   }
   return CORDE_OK;

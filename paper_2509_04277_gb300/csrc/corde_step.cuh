@@ -216,9 +216,10 @@ __device__ __forceinline__ void joint_torques(float4 qa, float4 qb, float4 uh, f
 // Segment forces between nodes a and b and the penalty torque on frame q (Eq. 8, and
 // Eq. 2 when the rod is extensible).  Penalty: E = 1/2 l0 Kp |t - d3|^2 gives the force
 // l0 Kp (d3 - (t . d3) t) / |e| on node b (opposite on a) and the torque l0 Kp d3 x t,
-// which in the body frame (d3 = e_z) is l0 Kp (-t_b.y, t_b.x, 0) with t_b = R(q)^T t.
+// which in the body frame (d3 = e_z) is l0 Kp (-t_b.y, t_b.x, 0) with t_b = R(q)^T t
+// (*t_body, if given).
 __device__ __forceinline__ void segment_forces(float3 ra, float3 rb, float4 q, const RodDev& R, bool extensible,
-                                               float3& fa, float3& fb, float3& tq) {
+                                               float3& fa, float3& fb, float3& tq, float3* t_body = nullptr) {
   const float3 e = rb - ra;
   const float ee = dot3(e, e);
   const float il = rsqrtf(ee);
@@ -236,6 +237,7 @@ __device__ __forceinline__ void segment_forces(float3 ra, float3 rb, float4 q, c
   }
   const float3 tb = rotate_inv(q, t);
   tq = f3(-R.lKp * tb.y, R.lKp * tb.x, 0.f);
+  if (t_body != nullptr) *t_body = tb;
 }
 
 // Impulse of one distance constraint (predictive: makes the segment length l0 after the

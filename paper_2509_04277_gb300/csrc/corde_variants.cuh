@@ -146,6 +146,19 @@ extern const ClusterVariant kClusterVariants[];
 extern const int kNumClusterVariants;
 constexpr int kMaxCluster = 16;
 
+// Overlapping warp tiles (corde_tile.cu): the latency form of the plain rod, with the results of
+// the <arith, *> layout.  One rod takes `blocks` blocks of `warps` warps, one tile a warp.
+struct TilePlan {
+  int per = 0;    // elements per lane (0: not a tile launch)
+  int arith = 0;  // elements per thread of the layout whose arithmetic it repeats
+  int blocks = 0, warps = 0;
+  int grid = 0;   // the blocks form a cooperative grid (one rod; a.grid_halo: its exchange buffers), not a cluster
+};
+constexpr int kTileMaxWarps = 8;           // warps per block
+int tile_count(int per, int n);            // tiles (warps) of a rod of n nodes
+int64_t tile_halo_bytes(int per, int n);   // global exchange buffers of a rod on a grid
+cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s);
+
 // Defined in the per-EPT instantiation units.
 extern const StepVariant kStepVariantsE2[];
 extern const int kNumStepVariantsE2;
