@@ -477,38 +477,25 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
   }
 }
 
+using TileFn = void (*)(const RodDev*, const int*, float4*, float4*, float4*, float4*, const float4*, const float4*,
+                        const float4*, int, float4*, int64_t, int, float4*, float4*);
+
 template <int PER, int ARITH>
-cudaError_t launch_t(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s) {
-  const int nt = 32 * p.warps;
-  if (p.warps > kTileMaxWarps) return cudaErrorInvalidValue;
-  const int smem = 2 * p.warps * Tile<PER>::kBuf * (int)sizeof(float4);
-  auto args = [&](auto kernel, int sm, int pdl, int cluster) {
-    if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e != cudaSuccess) return e;
-    }
-    if (cluster > 8) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-    }
-    return launch_kernel(kernel, dim3(n_rods * p.blocks), dim3(nt), sm, s, pdl, cluster, a.rods, a.work, a.x4, a.v4, a.q4,
-                         a.o4, a.u4, a.k4, a.drive, a.n_steps, a.traj, a.n_elem, p.blocks, a.grid_halo, a.pos_out);
-  };
-  if (p.grid) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_rods * p.blocks);
-    cfg.blockDim = dim3(nt);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tile_step_kernel<PER, ARITH, kTileGrid>, a.rods, a.work, a.x4, a.v4, a.q4, a.o4,
-                              a.u4, a.k4, a.drive, a.n_steps, a.traj, a.n_elem, p.blocks, a.grid_halo, a.pos_out);
-  }
-  if (p.blocks > 1) return args(tile_step_kernel<PER, ARITH, kTileCluster>, smem, a.pdl, p.blocks);
-  return args(tile_step_kernel<PER, ARITH, kTileBlock>, p.warps > 1 ? smem : 0, a.pdl, 0);
+TileFn tile_fn_t(const TilePlan& p) {
+  if (p.grid) return tile_step_kernel<PER, ARITH, kTileGrid>;
+  return p.blocks > 1 ? tile_step_kernel<PER, ARITH, kTileCluster> : tile_step_kernel<PER, ARITH, kTileBlock>;
+}
+TileFn tile_fn(const TilePlan& p) {
+  if (p.warps < 1 || p.warps > kTileMaxWarps) return nullptr;
+  if (p.per == 4 && p.arith == 4) return tile_fn_t<4, 4>(p);
+  if (p.per == 4 && p.arith == 2) return tile_fn_t<4, 2>(p);
+  if (p.per == 2 && p.arith == 4) return tile_fn_t<2, 4>(p);
+  if (p.per == 2 && p.arith == 2) return tile_fn_t<2, 2>(p);
+  return nullptr;
+}
+int tile_smem(const TilePlan& p, int warps) {
+  return p.grid || (p.blocks == 1 && warps == 1) ? 0
+                                                 : 2 * warps * (p.per == 4 ? Tile<4>::kBuf : Tile<2>::kBuf) * (int)sizeof(float4);
 }
 
 }  // namespace
@@ -518,12 +505,35 @@ int64_t tile_halo_bytes(int per, int n) {
   return (int64_t)2 * tile_count(per, n) * (per == 4 ? Tile<4>::kBuf : Tile<2>::kBuf) * (int64_t)sizeof(float4);
 }
 
+cudaError_t prepare_tile(const TilePlan& p) {
+  const TileFn fn = tile_fn(p);
+  if (fn == nullptr) return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
+  if (!p.grid) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(p, kTileMaxWarps));
+  if (e == cudaSuccess && p.blocks > 8 && !p.grid)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
 cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s) {
-  if (p.per == 4 && p.arith == 4) return launch_t<4, 4>(a, n_rods, p, s);
-  if (p.per == 4 && p.arith == 2) return launch_t<4, 2>(a, n_rods, p, s);
-  if (p.per == 2 && p.arith == 4) return launch_t<2, 4>(a, n_rods, p, s);
-  if (p.per == 2 && p.arith == 2) return launch_t<2, 2>(a, n_rods, p, s);
-  return cudaErrorInvalidValue;
+  const TileFn fn = tile_fn(p);
+  if (fn == nullptr) return cudaErrorInvalidValue;
+  const dim3 grid(n_rods * p.blocks), block(32 * p.warps);
+  if (!p.grid)
+    return launch_kernel(fn, grid, block, tile_smem(p, p.warps), s, a.pdl, p.blocks > 1 ? p.blocks : 0, a.rods, a.work, a.x4,
+                         a.v4, a.q4, a.o4, a.u4, a.k4, a.drive, a.n_steps, a.traj, a.n_elem, p.blocks, a.grid_halo,
+                         a.pos_out);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, a.rods, a.work, a.x4, a.v4, a.q4, a.o4, a.u4, a.k4, a.drive, a.n_steps, a.traj,
+                            a.n_elem, p.blocks, a.grid_halo, a.pos_out);
 }
 
 }  // namespace corde

@@ -157,6 +157,7 @@ struct TilePlan {
 constexpr int kTileMaxWarps = 8;           // warps per block
 int tile_count(int per, int n);            // tiles (warps) of a rod of n nodes
 int64_t tile_halo_bytes(int per, int n);   // global exchange buffers of a rod on a grid
+cudaError_t prepare_tile(const TilePlan& p);  // kernel attributes of the plan's launches, on the current device
 cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s);
 
 // Defined in the per-EPT instantiation units.

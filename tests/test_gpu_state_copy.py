@@ -1,0 +1,52 @@
+"""rod_get_state and rod_set_state between device buffers (one copy kernel), host buffers and
+device buffers that are not 16-byte aligned (a copy each): the same bytes, arrays that are
+not given untouched, and the inverse masses kept."""
+import numpy as np
+import pytest
+
+from paper_2509_04277_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+KEYS = ("pos4", "quat4", "vel4", "omega4")
+
+
+@pytest.fixture(scope="module")
+def corde(cuda):
+    from paper_2509_04277_gb300 import build, corde as C
+
+    build.build()
+    C.load()
+    return C
+
+
+@pytest.mark.parametrize("given", [(1, 1, 1, 1), (0, 1, 1, 1), (1, 0, 0, 0), (0, 0, 0, 1)])
+@pytest.mark.parametrize("shift", [0, 1])  # floats off a 16-byte boundary
+@pytest.mark.parametrize("n", [2, 127, 128, 129, 700])
+def test_device_buffers(corde, n, shift, given):
+    import torch
+
+    b = corde.RodBatch([W.guidewire(n, seed=n), W.guidewire(3, seed=1)])
+    b.step(5)
+    host = b.state_numpy()
+    E = b.n_elem
+
+    def buffers(fill):
+        return [torch.full((4 * E + 4,), fill, device="cuda")[shift:shift + 4 * E] for _ in KEYS]
+
+    out = buffers(-7.0)
+    corde.rod_get_state(b.handle, *[o if g else None for o, g in zip(out, given)])
+    for o, g, k in zip(out, given, KEYS):
+        got = o.cpu().numpy().reshape(E, 4)
+        assert np.array_equal(got, host[k] if g else np.full((E, 4), -7.0, np.float32))
+    new = buffers(0.0)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    for t in new:
+        t.copy_(torch.rand(4 * E, generator=gen, device="cuda"))
+    corde.rod_set_state(b.handle, *[t if g else None for t, g in zip(new, given)])
+    after = b.state_numpy()
+    for t, g, k in zip(new, given, KEYS):
+        want = t.cpu().numpy().reshape(E, 4) if g else host[k]
+        if k == "pos4":
+            want = np.concatenate([want[:, :3], host[k][:, 3:]], axis=1)
+        assert np.array_equal(after[k], want)
+    b.close()
