@@ -124,6 +124,17 @@ int default_variant(int n) {
   return best;
 }
 
+// The block of `threads` threads (a multiple of 32) with four elements per thread, NULL if the
+// variants themselves are the smallest that hold it.
+const StepVariant* trimmed_variant(int threads) {
+  const std::pair<const StepVariant*, int> t[] = {
+      {kStepTrimA, kNumStepTrimA}, {kStepTrimB, kNumStepTrimB}, {kStepTrimC, kNumStepTrimC}};
+  for (const auto& g : t)
+    for (int i = 0; i < g.second; ++i)
+      if (g.first[i].nt == threads) return &g.first[i];
+  return nullptr;
+}
+
 struct Bin {
   int variant;  // block variant index, or cluster variant index when cluster > 0
   int count;
@@ -132,6 +143,8 @@ struct Bin {
                     // indexes kSelfVariants)
   int grid = 0;     // 1: the cluster variant's blocks form a cooperative grid
   float4* d_gh = nullptr;  // grid bins: the rods' global exchange slots
+  int n_max = 0;           // nodes of the bin's longest rod
+  const StepVariant* trim = nullptr;  // the smaller block that holds the bin's rods
   TilePlan tile;           // per > 0: launches without a mailbox run the tile kernel
   float4* d_tile_gh = nullptr;  // tiles on a cooperative grid: their exchange buffers
 };
@@ -472,8 +485,18 @@ void invalidate_graph(rod_handle h) {
 int build_bins(rod_handle h) {
   invalidate_graph(h);
   free_bins(h);
-  std::vector<std::tuple<int, int, int>> keys;  // (blocks per rod, variant, grid)
-  auto key_of = [&](int r) { return std::make_tuple(h->plan_cluster[r], h->plan[r], (int)h->plan_grid[r]); };
+  // Threads of the smallest block that holds the rod in its <4, *> variant.  Power-of-two
+  // blocks are on average 28 % idle warps for log-uniform lengths, which take issue slots in
+  // the constraint sweeps and keep other blocks off the SM.
+  auto trim_of = [&](int r) {
+    if (h->plan_cluster[r] != 0 || variants()[h->plan[r]].ept != 4) return 0;
+    const int t = ((h->n_nodes[r] + 3) / 4 + 31) / 32 * 32;
+    return t < variants()[h->plan[r]].nt && trimmed_variant(t) ? t : 0;
+  };
+  std::vector<std::tuple<int, int, int, int>> keys;  // (blocks per rod, variant, grid, trimmed threads)
+  auto key_of = [&](int r) {
+    return std::make_tuple(h->plan_cluster[r], h->plan[r], (int)h->plan_grid[r], trim_of(r));
+  };
   for (int r = 0; r < h->n_rods; ++r) {
     if (r < (int)h->paired.size() && h->paired[r]) continue;
     const auto k = key_of(r);
@@ -491,6 +514,9 @@ int build_bins(rod_handle h) {
       return (int64_t)h->n_nodes[a] * (7 + h->n_iters[a]) > (int64_t)h->n_nodes[b] * (7 + h->n_iters[b]);
     });
     Bin b{std::get<1>(k), (int)rods.size(), nullptr, std::get<0>(k), std::get<2>(k)};
+    b.trim = trimmed_variant(std::get<3>(k));
+    b.n_max = 0;
+    for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
     if (b.grid) {
@@ -499,8 +525,7 @@ int build_bins(rod_handle h) {
       CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
     }
     if (b.cluster >= 0) {
-      int nmax = 0;
-      for (int r : rods) nmax = std::max(nmax, h->n_nodes[r]);
+      const int nmax = b.n_max;
       const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
       b.tile = tile_plan(nmax, b.count, arith, &spare);
       if (b.tile.per) CK(prepare_tile(b.tile));
@@ -508,6 +533,8 @@ int build_bins(rod_handle h) {
     }
     h->bins.push_back(b);
   }
+  // the longest rods first: their blocks run longest
+  std::stable_sort(h->bins.begin(), h->bins.end(), [](const Bin& a, const Bin& b) { return a.n_max > b.n_max; });
   return CORDE_OK;
 }
 
@@ -561,7 +588,7 @@ int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const f
                                         std::to_string(v.nt) + ", cluster=" + std::to_string(b.cluster) +
                                         "): " + cudaGetErrorString(e));
     } else {
-      const StepVariant& v = variants()[b.variant];
+      const StepVariant& v = b.trim ? *b.trim : variants()[b.variant];
       cudaError_t e = v.launch(a, b.count, s);
       if (e != cudaSuccess)
         return fail(CORDE_ERR_CUDA, std::string("step launch (ept=") + std::to_string(v.ept) +

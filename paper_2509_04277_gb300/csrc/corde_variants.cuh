@@ -165,5 +165,9 @@ extern const StepVariant kStepVariantsE2[];
 extern const int kNumStepVariantsE2;
 extern const StepVariant kStepVariantsE4[];
 extern const int kNumStepVariantsE4;
+// Four elements per thread, thread counts between the powers of two (not plans of their own:
+// a bin of a <4, *> plan runs on the smallest of them that holds its rods).
+extern const StepVariant kStepTrimA[], kStepTrimB[], kStepTrimC[];
+extern const int kNumStepTrimA, kNumStepTrimB, kNumStepTrimC;
 
 }  // namespace corde
