@@ -228,6 +228,8 @@ struct corde_rods {
   struct PairBin {
     int ept, nt, count;
     int4* d_pairs;
+    bool two_way;   // some pair binds both ways
+    TilePlan tile;  // per > 0: launches without a mailbox run the tile kernel
   };
   std::vector<PairBin> pair_bins;
   // mailbox of running launches
@@ -684,7 +686,8 @@ int launch_all(rod_handle h, int n_steps, const float4* d, cudaStream_t s, const
     for (const auto& pb : h->pair_bins) {
       cudaStream_t sk = branches ? (*branches)[k] : s;
       ++k;
-      cudaError_t e = launch_pair(pb.ept, pb.nt, a, pb.d_pairs, pb.count, sk);
+      cudaError_t e = pb.tile.per && !mb ? launch_pair_tile(a, pb.d_pairs, pb.count, pb.tile, pb.two_way, sk)
+                                         : launch_pair(pb.ept, pb.nt, a, pb.d_pairs, pb.count, sk);
       if (e != cudaSuccess) return fail(CORDE_ERR_CUDA, std::string("pair launch: ") + cudaGetErrorString(e));
       ++launches;
     }
@@ -1434,7 +1437,20 @@ static int build_pair_bins(rod_handle h) {
         if (e == ept && t == nt) ps.push_back(p);
       }
       if (ps.empty()) continue;
-      corde_rods::PairBin pb{ept, nt, (int)ps.size(), nullptr};
+      corde_rods::PairBin pb{ept, nt, (int)ps.size(), nullptr, false, TilePlan()};
+      for (const int4& p : ps) pb.two_way |= p.z == 2;
+      // tiles of both rods while they find idle SMs (see tile_plan): four warps per block, up to
+      // eight over the largest cluster
+      int n_max = 0;
+      for (const int4& p : ps) n_max = std::max({n_max, h->n_nodes[p.x], h->n_nodes[p.y]});
+      const int K = pair_tile_count(n_max);
+      pb.tile.arith = ept;
+      pb.tile.blocks = std::min((K + 3) / 4, kMaxCluster);
+      pb.tile.warps = (K + pb.tile.blocks - 1) / pb.tile.blocks;
+      if (pb.tile.warps <= kTileMaxWarps && (int64_t)pb.tile.blocks * pb.count + h->n_rods <= h->sms) {
+        CK(prepare_pair_tile(pb.tile, pb.two_way));
+        pb.tile.per = 2;
+      }
       CK(cudaMalloc(&pb.d_pairs, ps.size() * sizeof(int4)));
       CK(cudaMemcpy(pb.d_pairs, ps.data(), ps.size() * sizeof(int4), cudaMemcpyHostToDevice));
       h->pair_bins.push_back(pb);

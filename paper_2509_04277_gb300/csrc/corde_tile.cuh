@@ -1,0 +1,405 @@
+// Building blocks of the tile kernels (corde_tile.cu, corde_pair_tile.cu): the part of a rod that
+// one warp steps, PER elements per lane, and the exchange of ghosts between a rod's tiles.
+#pragma once
+
+#include <cooperative_groups.h>
+#include <type_traits>
+
+#include "corde_step.cuh"
+#include "corde_variants.cuh"
+
+namespace corde {
+
+template <int PER>
+struct Tile {
+  static constexpr int G = PER == 4 ? 6 : 11;  // ghost lanes on each side
+  static constexpr int O = 32 - 2 * G;         // lanes a tile owns (the rod's ends own their G too)
+  static constexpr int B = PER * G;            // elements an exchange makes valid on each side
+  static constexpr int SLOTS = PER == 4 ? 13 : 7;    // float4 of a lane's state: 13 floats per element
+  static constexpr int VSLOTS = (3 * PER + 3) / 4;   // float4 of its velocities
+  static constexpr int kBuf = SLOTS * 32;            // float4 of a tile's exchange buffer
+  // tiles of Q lanes' worth of elements
+  __host__ __device__ static int count_lanes(int Q) { return Q <= 32 ? 1 : (Q - 32 + O - 1) / O + 1; }
+  // tiles of a rod of n nodes
+  __host__ __device__ static int count(int n) { return count_lanes((n + PER - 1) / PER); }
+};
+
+__device__ __forceinline__ float3 down3(float3 a) {
+  return f3(__shfl_down_sync(0xffffffffu, a.x, 1), __shfl_down_sync(0xffffffffu, a.y, 1),
+            __shfl_down_sync(0xffffffffu, a.z, 1));
+}
+__device__ __forceinline__ float3 up3(float3 a) {
+  return f3(__shfl_up_sync(0xffffffffu, a.x, 1), __shfl_up_sync(0xffffffffu, a.y, 1),
+            __shfl_up_sync(0xffffffffu, a.z, 1));
+}
+__device__ __forceinline__ float3 add_rn(float3 a, float3 b) {
+  return f3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z));
+}
+
+// Predicted offset of a constraint and its reciprocal length.
+__device__ __forceinline__ float3 offset_of(float3 e, float3 va, float3 vb, float dt, float& il) {
+  const float3 d = f3(__fmaf_rn(dt, __fsub_rn(vb.x, va.x), e.x), __fmaf_rn(dt, __fsub_rn(vb.y, va.y), e.y),
+                      __fmaf_rn(dt, __fsub_rn(vb.z, va.z), e.z));
+  il = rsqrtf(__fmaf_rn(d.x, d.x, __fmaf_rn(d.y, d.y, __fmul_rn(d.z, d.z))));
+  return d;
+}
+
+// A warp's part of a rod: elements e0 ... e0 + PER - 1 of each lane (e0 >= n: none), stepped with
+// the arithmetic of the <ARITH, *> layout.
+template <int PER, int ARITH>
+struct TileRod {
+  static constexpr bool FOLD = StepCache<ARITH>::kFold;
+  const RodDev R;
+  const int lane, e0, n;
+  float3 r[PER], v[PER], om[PER], uh[PER], kk[PER];
+  float4 q[PER];
+  float w[PER];
+  // launch constants of the constraints: segment s joins elements s and s + 1; the last one
+  // reaches into the next lane, and the lane's first element also ends the previous lane's last
+  // one (index PER)
+  float inv[PER + 1], ca[PER + 1], la[PER + 1], cb[PER + 1], lb[PER + 1];
+  float3 e_seg[PER], e_left;  // the step's segment vectors
+
+  __device__ __forceinline__ TileRod(const RodDev& R_, int lane_, int e0_, const float4* __restrict__ x4,
+                                     const float4* __restrict__ v4, const float4* __restrict__ q4,
+                                     const float4* __restrict__ o4, const float4* __restrict__ u4,
+                                     const float4* __restrict__ k4)
+      : R(R_), lane(lane_), e0(e0_), n(R_.n) {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const int i = e0 + e;
+      r[e] = v[e] = om[e] = uh[e] = kk[e] = zero3();
+      q[e] = make_float4(0.f, 0.f, 0.f, 1.f);
+      w[e] = 0.f;
+      if (i < n) {
+        const float4 a = x4[R.off + i];
+        r[e] = f3(a);
+        w[e] = a.w;
+        v[e] = f3(v4[R.off + i]);
+        q[e] = q4[R.off + i];
+        om[e] = f3(o4[R.off + i]);
+        uh[e] = f3(u4[R.off + i]);
+        kk[e] = f3(k4[R.off + i]);
+      }
+    }
+    const float w_next = __shfl_down_sync(0xffffffffu, w[0], 1), w_prev = __shfl_up_sync(0xffffffffu, w[PER - 1], 1);
+#pragma unroll
+    for (int s = 0; s <= PER; ++s) {
+      const int j = s < PER ? e0 + s : e0 - 1;  // the segment's index in the rod
+      const float wa = s < PER ? w[s % PER] : w_prev, wb = s + 1 < PER ? w[(s + 1) % PER] : (s < PER ? w_next : w[0]);
+      const bool here = s < PER - 1 || (s == PER - 1 ? lane < 31 : lane > 0 && j >= 0);
+      inv[s] = inv_dt_wsum(here && j + 1 <= n - 1, wa, wb, R.dt);
+      ca[s] = wa * inv[s];
+      cb[s] = wb * inv[s];
+      la[s] = R.l0 * ca[s];
+      lb[s] = R.l0 * cb[s];
+    }
+    e_left = zero3();
+  }
+
+  // one distance constraint of the lane; segments PER - 1 and PER belong half to the
+  // neighbouring lanes, which compute the same impulse for their own half
+  __device__ __forceinline__ void constrain(int s, float3 es, float3 va, float3 vb, float3* pa, float3* pb) const {
+    float il;
+    const float3 d = offset_of(es, va, vb, R.dt, il);
+    if constexpr (FOLD) {
+      if (pa != nullptr) {
+        const float sa = -__fmaf_rn(la[s], il, -ca[s]);
+        *pa = f3(__fmaf_rn(sa, d.x, va.x), __fmaf_rn(sa, d.y, va.y), __fmaf_rn(sa, d.z, va.z));
+      }
+      if (pb != nullptr) {
+        const float sb = __fmaf_rn(lb[s], il, -cb[s]);
+        *pb = f3(__fmaf_rn(sb, d.x, vb.x), __fmaf_rn(sb, d.y, vb.y), __fmaf_rn(sb, d.z, vb.z));
+      }
+    } else {
+      const float sc = __fmul_rn(__fmaf_rn(R.l0, il, -1.f), inv[s]);
+      const float3 gi = f3(__fmul_rn(sc, d.x), __fmul_rn(sc, d.y), __fmul_rn(sc, d.z));
+      if (pa != nullptr) {
+        const float wa = w[s % PER];
+        *pa = f3(__fmaf_rn(-wa, gi.x, va.x), __fmaf_rn(-wa, gi.y, va.y), __fmaf_rn(-wa, gi.z, va.z));
+      }
+      if (pb != nullptr) {
+        const float wb = s < PER ? w[(s + 1) % PER] : w[0];
+        *pb = f3(__fmaf_rn(wb, gi.x, vb.x), __fmaf_rn(wb, gi.y, vb.y), __fmaf_rn(wb, gi.z, vb.z));
+      }
+    }
+  }
+
+  // Forces, their integration into the velocities, the frames, and the constraint geometry.
+  __device__ __forceinline__ void forces(float3 v_drive, float3 w_drive) {
+    const bool inext = (R.flags & F_INEXT) != 0, clamp = (R.flags & F_CLAMP) != 0;
+    const float dt = R.dt, half_dt = 0.5f * dt;
+    // ---- elastic forces and torques
+    float3 F[PER], tau[PER], Fc[PER + 1], Tc[PER + 1];
+#pragma unroll
+    for (int e = 0; e < PER; ++e) F[e] = tau[e] = zero3();
+#pragma unroll
+    for (int e = 0; e <= PER; ++e) Fc[e] = Tc[e] = zero3();
+    const float3 r_next = down3(r[0]), r_prev = up3(r[PER - 1]);
+    const float4 q_next = make_float4(__shfl_down_sync(0xffffffffu, q[0].x, 1), __shfl_down_sync(0xffffffffu, q[0].y, 1),
+                                      __shfl_down_sync(0xffffffffu, q[0].z, 1), __shfl_down_sync(0xffffffffu, q[0].w, 1));
+    auto joint_and_segment = [&](int e, float4 qb, float3 rb) {
+      const int j = e0 + e;
+      const bool carry = (e + 1) % (ARITH < PER ? ARITH : PER) == 0;  // to another lane, or a thread boundary of the layout
+      if (j <= n - 3) {
+        float3 ta, tb;
+        joint_torques(q[e], qb, make_float4(uh[e].x, uh[e].y, uh[e].z, 0.f), make_float4(kk[e].x, kk[e].y, kk[e].z, 0.f),
+                      R.two_over_l, ta, tb);
+        tau[e] += ta;
+        if (!carry) {
+          tau[(e + 1) % PER] += tb;
+        } else {
+          Tc[e + 1] = tb;
+        }
+      }
+      if (j <= n - 2) {
+        float3 fa, fb, tq;
+        segment_forces(r[e], rb, q[e], R, !inext, fa, fb, tq);
+        F[e] += fa;
+        tau[e] += tq;
+        if (!carry) {
+          F[(e + 1) % PER] += fb;
+        } else {
+          Fc[e + 1] = fb;
+        }
+      }
+    };
+    if constexpr (ARITH <= PER) {
+#pragma unroll
+      for (int e = 0; e < PER; ++e)
+        joint_and_segment(e, e + 1 < PER ? q[(e + 1) % PER] : q_next, e + 1 < PER ? r[(e + 1) % PER] : r_next);
+      Fc[0] = up3(Fc[PER]);
+      Tc[0] = up3(Tc[PER]);
+      if (lane == 0) Fc[0] = Tc[0] = zero3();
+    } else {
+      // two lanes make a thread of the <4, *> layout: the first element of the second lane
+      // takes the previous element's contribution before its own, the first lane's after
+      static_assert(ARITH <= PER || (PER == 2 && ARITH == 4), "tile layouts");
+      float3 ta = zero3(), fa = zero3(), fb, tq, tb = zero3();
+      if (e0 <= n - 3)
+        joint_torques(q[0], q[1], make_float4(uh[0].x, uh[0].y, uh[0].z, 0.f), make_float4(kk[0].x, kk[0].y, kk[0].z, 0.f),
+                      R.two_over_l, ta, tau[1]);
+      if (e0 <= n - 2) {
+        segment_forces(r[0], r[1], q[0], R, !inext, fa, fb, tq, &tb);
+        F[1] += fb;
+      }
+      joint_and_segment(1, q_next, r_next);
+      float3 Fi = up3(Fc[2]), Ti = up3(Tc[2]);
+      if (lane == 0) Fi = Ti = zero3();
+      if ((e0 >> 1) & 1) {
+        F[0] = Fi;
+        tau[0] = Ti;
+      } else {
+        Fc[0] = Fi;
+        Tc[0] = Ti;
+      }
+      F[0] = add_rn(F[0], fa);
+      tau[0] = add_rn(tau[0], ta);
+      // the penalty torque as the layouts fuse it (segment_forces' tq scaled and added)
+      tau[0] = f3(__fmaf_rn(-R.lKp, tb.y, tau[0].x), __fmaf_rn(R.lKp, tb.x, tau[0].y), tau[0].z);
+    }
+
+    // ---- constraint geometry
+#pragma unroll
+    for (int s = 0; s < PER; ++s)
+      e_seg[s] = safe_segment(inv[s], segment_vector(r[s], s + 1 < PER ? r[(s + 1) % PER] : r_next), R.l0);
+    e_left = safe_segment(inv[PER], segment_vector(r_prev, r[0]), R.l0);
+
+    // ---- force integration
+    auto integrate = [&](int e) {
+      const int i = e0 + e;
+      if (w[e] > 0.f) {
+        const float3 a = f3(w[e] * F[e].x + R.gx, w[e] * F[e].y + R.gy, w[e] * F[e].z + R.gz);
+        v[e] = R.damp * (v[e] + dt * a);
+      }
+      const bool frame_dynamic = (i <= n - 2) && !(clamp && i == 0);
+      if (frame_dynamic) {
+        const float3 o = om[e];
+        const float3 Jw = f3(R.J1 * o.x, R.J1 * o.y, R.J3 * o.z);
+        const float3 rhs = tau[e] - cross3(o, Jw);
+        const float3 on = f3(o.x + dt * R.Jinv1 * rhs.x, o.y + dt * R.Jinv1 * rhs.y, o.z + dt * R.Jinv3 * rhs.z);
+        om[e] = R.damp * on;
+      }
+    };
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      if (e % ARITH == 0) {  // (zero for a second lane of ARITH > PER)
+        F[e] = add_rn(F[e], Fc[e]);
+        tau[e] = add_rn(tau[e], Tc[e]);
+      }
+      integrate(e);
+    }
+    if (clamp && e0 == 0) {
+      v[0] = v_drive;
+      om[0] = w_drive;
+    }
+    // ---- frames
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      if (e0 + e <= n - 2) {
+        const float4 a = q[e];
+        const float3 o = om[e];
+        const float dx = a.w * o.x + a.y * o.z - a.z * o.y;
+        const float dy = a.w * o.y + a.z * o.x - a.x * o.z;
+        const float dz = a.w * o.z + a.x * o.y - a.y * o.x;
+        const float dwq = -(a.x * o.x + a.y * o.y + a.z * o.z);
+        const float4 b = make_float4(a.x + half_dt * dx, a.y + half_dt * dy, a.z + half_dt * dz, a.w + half_dt * dwq);
+        const float il = rsqrtf(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
+        q[e] = make_float4(b.x * il, b.y * il, b.z * il, b.w * il);
+      }
+    }
+  }
+
+  // One iteration of the distance constraints, red-black.
+  __device__ __forceinline__ void distance_iteration() {
+#pragma unroll
+    for (int s = 0; s < PER; s += 2) constrain(s, e_seg[s], v[s], v[s + 1], &v[s], &v[s + 1]);
+    const float3 vn = down3(v[0]), vp = up3(v[PER - 1]);
+#pragma unroll
+    for (int s = 1; s + 1 < PER; s += 2) constrain(s, e_seg[s], v[s], v[s + 1], &v[s], &v[s + 1]);
+    float3 v_last, v_first;
+    constrain(PER - 1, e_seg[PER - 1], v[PER - 1], vn, &v_last, nullptr);
+    constrain(PER, e_left, vp, v[0], nullptr, &v_first);
+    v[PER - 1] = v_last;
+    v[0] = v_first;
+  }
+
+  __device__ __forceinline__ void positions() {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) r[e] += R.dt * v[e];
+  }
+
+  // the lane's state as float4, and back
+  __device__ __forceinline__ void pack(float4* a) const {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      a[3 * e] = make_float4(r[e].x, r[e].y, r[e].z, v[e].x);
+      a[3 * e + 1] = make_float4(v[e].y, v[e].z, om[e].x, om[e].y);
+      a[3 * e + 2] = q[e];
+    }
+    a[3 * PER] = make_float4(om[0].z, om[1].z, om[PER - 2].z, om[PER - 1].z);
+  }
+  __device__ __forceinline__ void unpack(const float4* a) {
+    const float oz[4] = {a[3 * PER].x, a[3 * PER].y, a[3 * PER].z, a[3 * PER].w};
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      r[e] = f3(a[3 * e]);
+      v[e] = f3(a[3 * e].w, a[3 * e + 1].x, a[3 * e + 1].y);
+      q[e] = a[3 * e + 2];
+      om[e] = f3(a[3 * e + 1].z, a[3 * e + 1].w, oz[e]);
+    }
+  }
+  __device__ __forceinline__ void pack_v(float4* a) const {
+    constexpr int VS = Tile<PER>::VSLOTS;
+    float f[4 * VS];
+    f[4 * VS - 1] = f[4 * VS - 2] = 0.f;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      f[3 * e] = v[e].x;
+      f[3 * e + 1] = v[e].y;
+      f[3 * e + 2] = v[e].z;
+    }
+#pragma unroll
+    for (int s = 0; s < VS; ++s) a[s] = make_float4(f[4 * s], f[4 * s + 1], f[4 * s + 2], f[4 * s + 3]);
+  }
+  __device__ __forceinline__ void unpack_v(const float4* a) {
+    constexpr int VS = Tile<PER>::VSLOTS;
+    float f[4 * VS];
+#pragma unroll
+    for (int s = 0; s < VS; ++s) {
+      f[4 * s] = a[s].x;
+      f[4 * s + 1] = a[s].y;
+      f[4 * s + 2] = a[s].z;
+      f[4 * s + 3] = a[s].w;
+    }
+#pragma unroll
+    for (int e = 0; e < PER; ++e) v[e] = f3(f[3 * e], f[3 * e + 1], f[3 * e + 2]);
+  }
+
+  __device__ __forceinline__ void store(float4* __restrict__ x4, float4* __restrict__ v4, float4* __restrict__ q4,
+                                        float4* __restrict__ o4, float4* __restrict__ pos_out) const {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const int i = e0 + e;
+      if (i < n) {
+        x4[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
+        v4[R.off + i] = make_float4(v[e].x, v[e].y, v[e].z, 0.f);
+        q4[R.off + i] = q[e];
+        o4[R.off + i] = make_float4(om[e].x, om[e].y, om[e].z, 0.f);
+        if (pos_out != nullptr) pos_out[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
+      }
+    }
+  }
+};
+
+// How a rod's tiles exchange: the block's shared memory and barrier; the shared memory of a
+// cluster's blocks and its barrier; global memory and a grid sync.
+enum TileSync { kTileBlock, kTileCluster, kTileGrid };
+
+// A warp's place among the K tiles of a rod (or pair): tile k holds lanes k O ... k O + 31 of it.
+// BUF: float4 of a tile's exchange buffer, of which there are two, used in turn.
+template <int PER, int SYNC, int BUF>
+struct TileLink {
+  bool owned;               // the tile owns the lane's elements
+  float4* mine;             // where the lane publishes
+  const float4* theirs;     // where a ghost lane's owner publishes (NULL: not a ghost)
+  int64_t stride;           // from one buffer to the other
+  int parity = 0;
+
+  // Q: lanes of the whole rod; smem: the block's buffers, or gh: the grid's
+  __device__ __forceinline__ TileLink(int k, int K, int W, int lane, int Q, float4* smem, float4* gh) {
+    using T = Tile<PER>;
+    const bool active = k < K;
+    const int g = k * T::O + lane, wid = threadIdx.x >> 5;
+    owned = active && (k == 0 || lane >= T::G) && (k == K - 1 || lane < 32 - T::G);
+    mine = SYNC == kTileGrid ? gh + (int64_t)k * BUF + lane : smem + wid * BUF + lane;
+    stride = (int64_t)(SYNC == kTileGrid ? K : W) * BUF;
+    theirs = nullptr;
+    if (active && !owned && g < Q) {
+      const int ok = min(max((g - T::G) / T::O, 0), K - 1);  // the tile that owns lane g
+      const int ol = g - ok * T::O;
+      if constexpr (SYNC == kTileGrid) {
+        theirs = gh + (int64_t)ok * BUF + ol;
+      } else if constexpr (SYNC == kTileCluster) {
+        theirs = cooperative_groups::this_cluster().map_shared_rank(smem + (ok % W) * BUF + ol, ok / W);
+      } else {
+        theirs = smem + ok * BUF + ol;
+      }
+    }
+  }
+  __device__ __forceinline__ void barrier() const {
+    if constexpr (SYNC == kTileGrid) {
+      cooperative_groups::this_grid().sync();
+    } else if constexpr (SYNC == kTileCluster) {
+      cooperative_groups::this_cluster().sync();
+    } else {
+      __syncthreads();
+    }
+  }
+  // ghost lanes receive the N float4 of the lane that owns their elements (true for them)
+  template <int N>
+  __device__ __forceinline__ bool trade(float4 (&a)[N]) {
+    static_assert(N * 32 <= BUF, "exchange buffer");
+    if (owned) {
+      float4* m = mine + parity * stride;
+#pragma unroll
+      for (int s = 0; s < N; ++s) {
+        if constexpr (SYNC == kTileGrid) __stcg(m + s * 32, a[s]);
+        else m[s * 32] = a[s];
+      }
+    }
+    barrier();
+    if (theirs != nullptr) {
+      const float4* p = theirs + parity * stride;
+#pragma unroll
+      for (int s = 0; s < N; ++s) {
+        if constexpr (SYNC == kTileGrid) a[s] = __ldcg(p + s * 32);
+        else a[s] = p[s * 32];
+      }
+    }
+    parity ^= 1;
+    return theirs != nullptr;
+  }
+};
+
+}  // namespace corde
