@@ -541,8 +541,10 @@ int build_bins(rod_handle h) {
 }
 
 int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* drive, cudaStream_t s,
-                float4* traj = nullptr, const MailboxDev* mb = nullptr) {
+                float4* traj = nullptr, const MailboxDev* mb = nullptr, float4* ckpt = nullptr, int ckpt_every = 1) {
   StepArgs a = {};
+  a.ckpt = ckpt;
+  a.ckpt_every = ckpt_every;
   a.rods = h->d_rods;
   a.x4 = h->d_x;
   a.v4 = h->d_v;
@@ -568,6 +570,11 @@ int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const f
       if (e != cudaSuccess)
         return fail(CORDE_ERR_CUDA, std::string("tile step launch (blocks=") + std::to_string(b.tile.blocks) +
                                         ", warps=" + std::to_string(b.tile.warps) + "): " + cudaGetErrorString(e));
+    } else if (ckpt) {
+      const StepVariant& v = variants()[b.variant];
+      cudaError_t e = launch_rollout(v.nt, a, b.count, s);
+      if (e != cudaSuccess)
+        return fail(CORDE_ERR_CUDA, "rollout launch (nt=" + std::to_string(v.nt) + "): " + cudaGetErrorString(e));
     } else if (b.cluster < 0) {
       const StepVariant& v = kSelfVariants[b.variant];
       cudaError_t e = v.launch(a, b.count, s);
@@ -1537,7 +1544,11 @@ int rod_rollout(rod_handle h, int n_steps, int ckpt_every, float* pos_traj, void
     if (int rc = build_adjoint_bins(h)) return rc;
   const std::vector<Bin>& bins = adj ? h->adj_bins : h->bins;
   int launches = 0;
-  for (int seg = 0; seg < n_seg; ++seg) {
+  if (adj) {  // all segments in one launch per bin
+    if (int rc = launch_bins(h, bins, n_steps, h->d_drive, s, traj, nullptr, h->d_ckpt, ckpt_every)) return rc;
+    launches = h->last_launches;
+  }
+  for (int seg = 0; seg < n_seg && !adj; ++seg) {
     float4* ck = h->d_ckpt + (size_t)seg * 4 * E;
     Copy4 c = {{h->d_x, h->d_v, h->d_q, h->d_o}, {ck, ck + E, ck + 2 * E, ck + 3 * E}};
     CK(launch_copy4(c, E, 0, s));

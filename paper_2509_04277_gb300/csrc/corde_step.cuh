@@ -933,15 +933,36 @@ struct RodMailbox {
   }
 };
 
+// Checkpoints of a rollout: the state before every `every`-th step, [n][4][n_elem] float4
+// (positions and masses, velocities, frames, angular velocities).
+struct CkptDev {
+  float4* ckpt;
+  int every;
+};
+template <int EPT>
+__device__ __forceinline__ void put_checkpoint(const CkptDev& c, int step, const RodDev& R, int e0, int64_t n_elem,
+                                               const float3 (&r)[EPT], const float3 (&v)[EPT], const float4 (&q)[EPT],
+                                               const float3 (&om)[EPT], const float (&w)[EPT]) {
+  float4* ck = c.ckpt + (int64_t)(step / c.every) * 4 * n_elem + R.off + e0;
+#pragma unroll
+  for (int e = 0; e < EPT; ++e)
+    if (e0 + e < R.n) {
+      ck[e] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
+      ck[n_elem + e] = make_float4(v[e].x, v[e].y, v[e].z, 0.f);
+      ck[2 * n_elem + e] = q[e];
+      ck[3 * n_elem + e] = make_float4(om[e].x, om[e].y, om[e].z, 0.f);
+    }
+}
+
 // The launch of one rod by the threads described by H: load, n_steps steps (with the
-// optional trajectory output and mailbox), store.
-template <int EPT, int NT, class Halo>
+// optional trajectory output and mailbox; CKPT: a rollout's checkpoints), store.
+template <int EPT, int NT, bool CKPT = false, class Halo>
 __device__ __forceinline__ void run_rod(const RodDev& R, const Halo& H, const int rid, const float4* __restrict__ x4in,
                                         float4* __restrict__ x4, float4* __restrict__ v4, float4* __restrict__ q4,
                                         float4* __restrict__ o4, const float4* __restrict__ u4,
                                         const float4* __restrict__ k4, const float4* __restrict__ drive, int n_steps,
                                         float4* __restrict__ traj, int64_t n_elem, const MailboxDev& mb, float4* smem,
-                                        float4* __restrict__ pos_out) {
+                                        float4* __restrict__ pos_out, const CkptDev& ckpt = CkptDev{nullptr, 1}) {
   float4* par_u = smem;
   float4* par_k = smem + EPT * NT;
   float4* halo = smem + 2 * EPT * NT;
@@ -962,6 +983,9 @@ __device__ __forceinline__ void run_rod(const RodDev& R, const Halo& H, const in
   StepCache<EPT> sc;  // launch constants of the step (filled on the first step)
   for (int step = 0; step < n_steps; ++step) {
     if (box.before_step(H, step, v_drive, w_drive)) break;
+    if constexpr (CKPT) {
+      if (step % ckpt.every == 0) put_checkpoint<EPT>(ckpt, step, R, e0, n_elem, r, v, q, om, w);
+    }
     step_body<EPT, NT, false>(R, H, r, v, q, om, w, par_u, par_k, halo, xc, sc, v_drive, w_drive, nullptr, nullptr);
     if (traj != nullptr) {
 #pragma unroll
@@ -1001,6 +1025,22 @@ step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, float
   const RodDev R = rods[rid];
   const BlockHalo<NT, NT, EPT == 2> H{(int)threadIdx.x};
   run_rod<EPT, NT>(R, H, rid, x4, x4, v4, q4, o4, u4, k4, drive, n_steps, traj, n_elem, mb, smem, pos_out);
+}
+
+// A whole recorded rollout in one launch: step_kernel with checkpoints.
+template <int EPT, int NT>
+__global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 512 / NT)
+rollout_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, float4* __restrict__ x4,
+               float4* __restrict__ v4, float4* __restrict__ q4, float4* __restrict__ o4, const float4* __restrict__ u4,
+               const float4* __restrict__ k4, const float4* __restrict__ drive, int n_steps, float4* __restrict__ traj,
+               int64_t n_elem, CkptDev ckpt) {
+  extern __shared__ float4 smem[];
+  pdl_begin();
+  const int rid = work[blockIdx.x];
+  const RodDev R = rods[rid];
+  const BlockHalo<NT, NT, EPT == 2> H{(int)threadIdx.x};
+  run_rod<EPT, NT, true>(R, H, rid, x4, x4, v4, q4, o4, u4, k4, drive, n_steps, traj, n_elem, MailboxDev{}, smem, nullptr,
+                         ckpt);
 }
 
 }  // namespace corde

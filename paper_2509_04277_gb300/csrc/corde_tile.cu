@@ -25,7 +25,7 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
                  float4* __restrict__ v4, float4* __restrict__ q4, float4* __restrict__ o4,
                  const float4* __restrict__ u4, const float4* __restrict__ k4, const float4* __restrict__ drive,
                  int n_steps, float4* __restrict__ traj, int64_t n_elem, int C, float4* __restrict__ gh,
-                 float4* __restrict__ pos_out) {
+                 float4* __restrict__ pos_out, CkptDev ckpt) {
   using T = Tile<PER>;
   extern __shared__ float4 smem[];
   const int lane = threadIdx.x & 31, W = blockDim.x >> 5;
@@ -90,6 +90,8 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
       since = 0;
     }
     ++since;
+    if (ckpt.ckpt != nullptr && link.owned && step % ckpt.every == 0)
+      put_checkpoint<PER>(ckpt, step, R, rod.e0, n_elem, rod.r, rod.v, rod.q, rod.om, rod.w);
     if (active) rod.forces(v_drive, w_drive);
     if (inext) {
       if (n_iters <= kChunk || K == 1) {
@@ -135,7 +137,7 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
 }
 
 using TileFn = void (*)(const RodDev*, const int*, float4*, float4*, float4*, float4*, const float4*, const float4*,
-                        const float4*, int, float4*, int64_t, int, float4*, float4*);
+                        const float4*, int, float4*, int64_t, int, float4*, float4*, CkptDev);
 
 template <int PER, int ARITH>
 TileFn tile_fn_t(const TilePlan& p) {
@@ -179,7 +181,7 @@ cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaSt
   if (!p.grid)
     return launch_kernel(fn, grid, block, tile_smem(p, p.warps), s, a.pdl, p.blocks > 1 ? p.blocks : 0, a.rods, a.work, a.x4,
                          a.v4, a.q4, a.o4, a.u4, a.k4, a.drive, a.n_steps, a.traj, a.n_elem, p.blocks, a.grid_halo,
-                         a.pos_out);
+                         a.pos_out, CkptDev{a.ckpt, a.ckpt_every});
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -190,7 +192,7 @@ cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaSt
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, fn, a.rods, a.work, a.x4, a.v4, a.q4, a.o4, a.u4, a.k4, a.drive, a.n_steps, a.traj,
-                            a.n_elem, p.blocks, a.grid_halo, a.pos_out);
+                            a.n_elem, p.blocks, a.grid_halo, a.pos_out, CkptDev{a.ckpt, a.ckpt_every});
 }
 
 }  // namespace corde

@@ -24,6 +24,8 @@ struct StepArgs {
   int4* self_stats;  // self-collision statistics per rod (corde_self.cu), or NULL
   unsigned char* self_skin;  // self-collision skin lists kept between launches (corde_self.cu), or NULL
   float4* pos_out;   // optional: positions (r, w) after the launch, [n_elem] (device or mapped host)
+  float4* ckpt;      // rollouts: checkpoints every ckpt_every steps (see CkptDev), or NULL
+  int ckpt_every;
   float4* grid_halo; // rods on a cooperative grid: their global exchange slots
   int pdl;           // 1: launch with programmatic stream serialisation (the kernel may start
                      // before the stream's previous kernel ends; it waits in pdl_begin)
@@ -62,6 +64,8 @@ typedef cudaError_t (*StepLaunchFn)(const StepArgs& a, int n_blocks, cudaStream_
 // Loads the variant's kernel into the current context now (cudaFuncGetAttributes), so
 // that its first launch does not load the module (lazy loading takes device memory).
 typedef cudaError_t (*StepPreloadFn)();
+// A rollout with its checkpoints on the two-element block of nt threads (a.ckpt set).
+cudaError_t launch_rollout(int nt, const StepArgs& a, int n_blocks, cudaStream_t s);
 
 struct StepVariant {
   int ept;
