@@ -1509,7 +1509,8 @@ static int build_adjoint_bins(rod_handle h) {
     Bin b{v, (int)rods.size(), nullptr};
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
-    b.tile = tile_plan(2 * nt, b.count, 2, &spare);
+    for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
+    b.tile = tile_plan(b.n_max, b.count, 2, &spare);
     if (b.tile.per) CK(prepare_tile(b.tile));
     h->adj_bins.push_back(b);
   }
@@ -1613,8 +1614,26 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   std::vector<int> mode(h->adj_bins.size(), 0);
   std::vector<char> compact(h->adj_bins.size(), 0);
   std::vector<char> pipe(h->adj_bins.size(), 0);
-  size_t sweep_need = 0;
+  // Tiles: the rods of a bin spread over SMs of their own (one warp per SM partition), when the
+  // records and states of every step fit the budget and the iterations the tiles' ghosts
+  std::vector<int> tile_blocks(h->adj_bins.size(), 0);
+  size_t sweep_need = 0, seg_need = 0;
+  int spare = sms - h->n_rods;
+  for (size_t i = 0; i < h->adj_bins.size() && h->adj_pipe && iters <= kAdjointTileIters; ++i) {
+    const Bin& b = h->adj_bins[i];
+    const int blocks = (tile_count(2, b.n_max) + 3) / 4;
+    const size_t rec = (size_t)h->ro_steps * b.count * 2 * iters * 3 * adjoint_tile_npad(b.n_max) / 4;  // float4
+    const size_t states = (size_t)(h->ro_steps + 1) * 4 * E;
+    if (spare < 0 || (blocks - 1) * b.count > spare ||
+        (long long)((rec + states) * sizeof(float4)) > h->adj_record_budget)
+      continue;
+    spare -= (blocks - 1) * b.count;
+    tile_blocks[i] = blocks;
+    sweep_need = std::max(sweep_need, rec);
+    seg_need = states;
+  }
   for (size_t i = 0; i < h->adj_bins.size(); ++i) {
+    if (tile_blocks[i]) continue;
     const Bin& b = h->adj_bins[i];
     const int nt = variants()[b.variant].nt;
     const bool prefer_compact = b.count > sms;
@@ -1654,8 +1673,8 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   }
   const bool any_record = sweep_need > 0;
   const bool any_pipe = std::find(pipe.begin(), pipe.end(), 1) != pipe.end();
-  if (int rc = ensure_capacity(&h->d_seg, &h->seg_cap, (K + (any_record ? 1 : 0)) * (any_pipe ? 2 : 1) * 4 * E))
-    return rc;
+  seg_need = std::max(seg_need, (K + (any_record ? 1 : 0)) * (any_pipe ? 2 : 1) * 4 * E);
+  if (int rc = ensure_capacity(&h->d_seg, &h->seg_cap, seg_need)) return rc;
   if (any_record) {
     if (int rc = ensure_capacity(&h->d_sweep_rec, &h->sweep_rec_cap, sweep_need)) return rc;
   }
@@ -1681,6 +1700,40 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   for (size_t i = 0; i < h->adj_bins.size(); ++i) {
     const Bin& b = h->adj_bins[i];
     const int nt = variants()[b.variant].nt;
+    if (tile_blocks[i]) {
+      const int blocks = tile_blocks[i], warps = (tile_count(2, b.n_max) + blocks - 1) / blocks;
+      AdjointTileArgs t = {};
+      t.rods = a.rods;
+      t.work = b.d_work;
+      t.n_rods = b.count;
+      t.blocks = blocks;
+      t.ckpt = a.ckpt;
+      t.states = h->d_seg;
+      t.rec = reinterpret_cast<float*>(h->d_sweep_rec);
+      t.rec_iters = iters;
+      t.npad = adjoint_tile_npad(b.n_max);
+      t.u4 = a.u4;
+      t.k4 = a.k4;
+      t.drive = a.drive;
+      t.dLdpos = a.dLdpos;
+      t.n_steps = a.n_steps;
+      t.ckpt_every = a.ckpt_every;
+      t.n_elem = E;
+      t.dpos0 = a.dpos0;
+      t.dvel0 = a.dvel0;
+      t.dquat0 = a.dquat0;
+      t.domega0 = a.domega0;
+      t.dK = a.dK;
+      t.duhat = a.duhat;
+      if (blocks * b.count >= h->adj_info[3]) {
+        const int info[7] = {2, 32 * warps, 1, blocks * b.count, sms, 0, 1};
+        std::copy(info, info + 7, h->adj_info);
+      }
+      cudaError_t e = launch_adjoint_tile(t, warps, s);
+      if (e != cudaSuccess) return fail(CORDE_ERR_CUDA, std::string("adjoint tile launch: ") + cudaGetErrorString(e));
+      launches += 2;
+      continue;
+    }
     int smem = adjoint_smem_bytes(nt, iters, mode[i], compact[i] != 0);
     // pipelined: shared memory of more than half an SM keeps the cluster's two blocks on
     // two SMs

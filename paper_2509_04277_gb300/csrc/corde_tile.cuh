@@ -251,9 +251,11 @@ struct TileRod {
   }
 
   // One iteration of the distance constraints, red-black.
-  __device__ __forceinline__ void distance_iteration() {
+  __device__ __forceinline__ void even_sweep() {
 #pragma unroll
     for (int s = 0; s < PER; s += 2) constrain(s, e_seg[s], v[s], v[s + 1], &v[s], &v[s + 1]);
+  }
+  __device__ __forceinline__ void odd_sweep() {
     const float3 vn = down3(v[0]), vp = up3(v[PER - 1]);
 #pragma unroll
     for (int s = 1; s + 1 < PER; s += 2) constrain(s, e_seg[s], v[s], v[s + 1], &v[s], &v[s + 1]);
@@ -262,6 +264,10 @@ struct TileRod {
     constrain(PER, e_left, vp, v[0], nullptr, &v_first);
     v[PER - 1] = v_last;
     v[0] = v_first;
+  }
+  __device__ __forceinline__ void distance_iteration() {
+    even_sweep();
+    odd_sweep();
   }
 
   __device__ __forceinline__ void positions() {
@@ -376,6 +382,18 @@ struct TileLink {
       __syncthreads();
     }
   }
+  // the barrier of an exchange: it orders the tiles' shared-memory buffers (global memory on a grid)
+  // and nothing else.  The full cluster barrier also waits for a block's global accesses in
+  // flight, the adjoint's prefetches above all.
+  __device__ __forceinline__ void meet() const {
+    if constexpr (SYNC == kTileCluster) {
+      asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+      barrier();
+    }
+  }
   // ghost lanes receive the N float4 of the lane that owns their elements (true for them)
   template <int N>
   __device__ __forceinline__ bool trade(float4 (&a)[N]) {
@@ -388,7 +406,7 @@ struct TileLink {
         else m[s * 32] = a[s];
       }
     }
-    barrier();
+    meet();
     if (theirs != nullptr) {
       const float4* p = theirs + parity * stride;
 #pragma unroll

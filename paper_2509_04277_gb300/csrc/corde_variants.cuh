@@ -122,6 +122,27 @@ cudaError_t adjoint_occupancy(int nt, int mode, bool compact, int smem, int* blo
 cudaError_t launch_adjoint_pipe(int nt, const AdjointArgs& a, int n_rods, int smem, cudaStream_t s);
 constexpr int kAdjointMaxNodes = 512;
 
+// The adjoint on warp tiles (corde_adjoint_tile.cu): `blocks` blocks per rod, at most
+// kAdjointTileIters constraint iterations.
+struct AdjointTileArgs {
+  const RodDev* rods;
+  const int* work;
+  int n_rods, blocks;
+  const float4* ckpt;   // [n_ckpt][4][n_elem]
+  float4* states;       // scratch [n_steps + 1][4][n_elem]: the state before every step (and after the last)
+  float* rec;           // scratch [n_steps][n_rods][2 rec_iters][3][npad]: velocities before every half-sweep
+  int rec_iters, npad;
+  const float4 *u4, *k4, *drive;
+  const float4* dLdpos;  // [n_steps][n_elem] or NULL
+  int n_steps, ckpt_every;
+  int64_t n_elem;
+  float4 *dpos0, *dvel0, *dquat0, *domega0, *dK, *duhat;
+};
+constexpr int kAdjointTileIters = 10;
+int adjoint_tile_npad(int n);  // floats of a record row of rods of at most n nodes
+// Records all segments, then reverses them (two launches).
+cudaError_t launch_adjoint_tile(const AdjointTileArgs& a, int warps, cudaStream_t s);
+
 // Rods with self-collision (corde_self.cu): one rod per block, at most 1024 nodes.
 extern const StepVariant kSelfVariants[];
 extern const int kNumSelfVariants;

@@ -1,0 +1,86 @@
+"""The adjoint on warp tiles against the one-block reverse kernel: the same gradients bit for bit
+for lengths at the tiles' edges, every iteration count the ghosts hold, short last segments,
+extensible rods and several rods of different lengths; beyond (more iterations, a budget that
+the records do not fit) the block kernels run."""
+import numpy as np
+import pytest
+
+from paper_2509_04277_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def corde(cuda):
+    from paper_2509_04277_gb300 import build, corde as C
+
+    build.build()
+    C.load()
+    return C
+
+
+def _grads(corde, rods, n_steps, every, tiles, budget=None):
+    import torch
+
+    b = corde.RodBatch(rods)
+    b.set_adjoint_pipeline(tiles)
+    if budget is not None:
+        b.set_adjoint_record_budget(budget)
+    drive = np.zeros((len(rods), 8), np.float32)
+    drive[:, 0], drive[:, 6] = 0.02, 1.0
+    b.set_input(drive)
+    traj = b.rollout(n_steps, every)
+    g = torch.zeros_like(traj)
+    g[:, :, :3] = 1e-2 * torch.cos(traj[:, :, :3] * 23.0)
+    out = {k: v.cpu().numpy() for k, v in b.adjoint(g).items()}
+    out["traj"] = traj.cpu().numpy()
+    info = corde.rod_adjoint_info(b.handle)
+    b.close()
+    return out, info
+
+
+def _same(corde, rods, n_steps=7, every=3):
+    (a, ia), (c, ic) = (_grads(corde, rods, n_steps, every, t) for t in (True, False))
+    assert ia["pipelined"] and not ic["pipelined"]
+    for k in a:
+        assert np.isfinite(a[k]).all(), k
+        np.testing.assert_array_equal(a[k], c[k], err_msg=k)
+
+
+@pytest.mark.parametrize("n", [2, 3, 63, 64, 65, 84, 85, 104, 144, 145, 256, 511, 512])
+def test_lengths(corde, n):
+    rod = W.adjoint_rod(n, seed=n) if n > 2 else W.guidewire(2, seed=2)
+    _same(corde, [rod])
+
+
+@pytest.mark.parametrize("iters", [0, 1, 2, 9, 10])
+def test_iterations(corde, iters):
+    rod = W.adjoint_rod(150, seed=iters)
+    rod.n_iters = iters
+    _same(corde, [rod])
+
+
+@pytest.mark.parametrize("n_steps,every", [(1, 1), (4, 1), (5, 9), (9, 4)])
+def test_segments(corde, n_steps, every):
+    _same(corde, [W.adjoint_rod(100, seed=1)], n_steps, every)
+
+
+def test_uneven_and_extensible_rods(corde):
+    rods = [W.adjoint_rod(n, seed=n) for n in (40, 300, 90, 301, 512)]
+    rods[2].n_iters = 4
+    _same(corde, rods)
+    _same(corde, [W.extensible_pendulum(100, seed=3)])
+
+
+def test_where_the_tiles_end(corde):
+    rod = W.adjoint_rod(100, seed=5)
+    rod.n_iters = 11
+    a, ia = _grads(corde, [rod], 6, 3, True)
+    c, _ = _grads(corde, [rod], 6, 3, False)
+    assert all(np.array_equal(a[k], c[k]) for k in a)
+    assert ia["blocks"] == 2  # the two-block pipeline
+    rod.n_iters = 10
+    a, _ = _grads(corde, [rod], 6, 3, True)
+    c, ic = _grads(corde, [rod], 6, 3, True, budget=100000)  # one segment's records fit, all six steps' do not
+    assert ic["mode"] == "recompute" or ic["blocks"] <= 2
+    assert all(np.array_equal(a[k], c[k]) for k in a)
