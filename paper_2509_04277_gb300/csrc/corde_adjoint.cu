@@ -26,7 +26,7 @@ template <int NT>
 struct BlockNet {
   static constexpr bool kShared = false;  // (one exchange less on the chain)
   static constexpr int kUnroll = 2;       // iterations per block of code
-  const int t;
+  const int t, tn, tp;
   const float4 *par_u, *par_k;
   float4* halo;
   int& xc;
@@ -38,8 +38,8 @@ struct BlockNet {
   __device__ __forceinline__ float4 k(int e) const { return par_k[e * NT + t]; }
   __device__ __forceinline__ float3 rec(int slot, int e) const { return rec_get<2, NT>(sweep_v, slot, e, t); }
   // (in-range neighbour slots at the ends)
-  __device__ __forceinline__ float3 rec_next(int slot) const { return rec_get<2, NT>(sweep_v, slot, 0, min(t + 1, NT - 1)); }
-  __device__ __forceinline__ float3 rec_prev(int slot) const { return rec_get<2, NT>(sweep_v, slot, 1, max(t - 1, 0)); }
+  __device__ __forceinline__ float3 rec_next(int slot) const { return rec_get<2, NT>(sweep_v, slot, 0, tn); }
+  __device__ __forceinline__ float3 rec_prev(int slot) const { return rec_get<2, NT>(sweep_v, slot, 1, tp); }
   __device__ __forceinline__ float4* buffer() {
     float4* hb = halo + (xc & 1) * kHaloSlots * NT;
     ++xc;
@@ -297,7 +297,7 @@ adjoint_kernel(AdjointArgs a) {
           if constexpr (NBUF == 2) fetch(seg, s - 1, sweep_v + ((s - 1) & 1) * rec_stride);
           prefetch(s - 1);
         }
-        BlockNet<NT> net{t, par_u, par_k, halo, xc, sweep_v + (s % NBUF) * rec_stride};
+        BlockNet<NT> net{t, min(t + 1, NT - 1), max(t - 1, 0), par_u, par_k, halo, xc, sweep_v + (s % NBUF) * rec_stride};
         reverse_step<COMPACT>(R, net, r_in, q_in, om_in, w, om, q, nb, sc, rb, vb, qb, ob, Kb, ub);
         if constexpr (NBUF == 1) {
           if (s > 0) {
@@ -350,7 +350,7 @@ adjoint_kernel(AdjointArgs a) {
           for (int e = 0; e < EPT; ++e)
             if (e0 + e < R.n) rb[e] += g_s[e];
         }
-        BlockNet<NT> net{t, par_u, par_k, halo, xc, sweep_v};
+        BlockNet<NT> net{t, min(t + 1, NT - 1), max(t - 1, 0), par_u, par_k, halo, xc, sweep_v};
         reverse_step<COMPACT>(R, net, r_in, q_in, om_in, w, om, q, nb, sc, rb, vb, qb, ob, Kb, ub);
       }
     }
