@@ -149,16 +149,28 @@ struct Bin {
   float4* d_tile_gh = nullptr;  // tiles on a cooperative grid: their exchange buffers
 };
 
+// How much of the GPU a handle's rods leave free (see tile_plan).
+struct TileRoom {
+  int sms;
+  int spare;       // SMs beyond one per rod that no tile plan has taken yet
+  bool saturated;  // the rods' block kernels alone put more than two warps on every SM partition
+};
+
 // Tile plan of a bin of `count` rods of at most n nodes whose kernel layout has `arith`
-// elements per thread; per = 0 where the block, cluster or grid kernel runs.
-// The tiles repeat their ghosts' work (three times an element's at two elements per lane, 1.6
-// times at four), so they are for handles that leave SMs idle: every rod has one SM and the
-// tiles take from the `spare` others (which a tile plan reduces).  One warp per SM partition is fastest (512 nodes: 2.15 us/step at 4 warps
-// a block, 2.50 at 6, 2.59 at 8).
-// Two elements per lane shorten the chain of a step (512 nodes: 2.15 against 2.88 us/step at
-// four) and win up to seven warps a block over the largest cluster (2048 nodes: 2.73 against
-// 2.98); longer rods take four (5000 nodes: 3.02 on a cluster, 3.62 at two on a grid).
-TilePlan tile_plan(int n, int count, int arith, int* spare) {
+// elements per thread; per = 0 where the block, cluster or grid kernel runs.  Measured at 10 iterations:
+//  - Over several SMs while there are spare ones: the tiles repeat their ghosts' work (three times
+//    an element's at two elements per lane, 1.6 times at four).  One warp per SM partition is
+//    fastest (512 nodes: 2.15 us/step at 4 warps a block, 2.50 at 6, 2.59 at 8).  Two elements per
+//    lane shorten the chain of a step (512 nodes: 2.15 against 2.88 us/step at four) and win up
+//    to seven warps a block over the largest cluster (2048 nodes: 2.73 against 2.98); longer rods
+//    take four (5000 nodes: 3.02 on a cluster, 3.62 at two on a grid).
+//  - Otherwise in one block of up to four tiles, while all rods' tiles find two warps per SM
+//    partition: 608 rods of 128 / 200 nodes 2.40 / 3.54 us/step against 3.46 / 4.03 as blocks, 304 of
+//    360 nodes 3.45 against 4.44; with more rods the repeated work loses (400 of 256: 5.64 / 3.90).
+//  - A rod of one tile repeats nothing: shuffles beat shared memory at any load, with the
+//    registers of 16 warps per SM (4864 rods of 64 nodes 5.53 us/step against 6.98, of 128 nodes
+//    11.1 against 11.4).
+TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   TilePlan p;
   p.arith = arith;
   const int K2 = tile_count(2, n), K4 = tile_count(4, n);
@@ -168,15 +180,20 @@ TilePlan tile_plan(int n, int count, int arith, int* spare) {
   if (K > 8 * p.blocks) {
     // more tiles than a cluster holds: a cooperative grid, one block per SM
     p.grid = 1;
-    p.blocks = std::min(K, *spare + 1);
+    p.blocks = std::min(K, room->spare + 1);
   }
   p.warps = p.blocks > 0 ? (K + p.blocks - 1) / p.blocks : 0;
   const int64_t more = (int64_t)(p.blocks - 1) * count;
-  if (p.blocks < 1 || p.warps > kTileMaxWarps || (p.grid && count > 1) || *spare < 0 || more > *spare) {
-    p.per = 0;
-  } else {
-    *spare -= (int)more;
+  if (p.blocks >= 1 && p.warps <= kTileMaxWarps && !(p.grid && count > 1) && room->spare >= more) {
+    room->spare -= (int)more;
+    return p;
   }
+  p.grid = 0;
+  p.blocks = 1;
+  p.per = K2 == 1 ? 2 : 4;
+  p.warps = K2 == 1 ? 1 : K4;
+  p.full = K2 == 1 || (K4 == 1 && room->saturated);
+  if (p.full ? (K2 > 1 && arith != 4) : (room->saturated || K4 > 4 || count > 8 / K4 * room->sms)) p.per = 0;
   return p;
 }
 
@@ -484,6 +501,12 @@ void invalidate_graph(rod_handle h) {
   h->graph_steps = -1;
 }
 
+TileRoom tile_room(rod_handle h) {
+  int64_t warps = 0;
+  for (int r = 0; r < h->n_rods; ++r) warps += (h->n_nodes[r] + 127) / 128;
+  return TileRoom{h->sms, h->sms - h->n_rods, warps > 8 * (int64_t)h->sms};
+}
+
 int build_bins(rod_handle h) {
   invalidate_graph(h);
   free_bins(h);
@@ -505,7 +528,7 @@ int build_bins(rod_handle h) {
     if (std::find(keys.begin(), keys.end(), k) == keys.end()) keys.push_back(k);
   }
   std::sort(keys.begin(), keys.end());
-  int spare = h->sms - h->n_rods;
+  TileRoom room = tile_room(h);
   for (const auto& k : keys) {
     std::vector<int> rods;
     for (int r = 0; r < h->n_rods; ++r)
@@ -529,7 +552,7 @@ int build_bins(rod_handle h) {
     if (b.cluster >= 0) {
       const int nmax = b.n_max;
       const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
-      b.tile = tile_plan(nmax, b.count, arith, &spare);
+      b.tile = tile_plan(nmax, b.count, arith, &room);
       if (b.tile.per) CK(prepare_tile(b.tile));
       if (b.tile.per && b.tile.grid) CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
     }
@@ -1284,8 +1307,8 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         if (v.capacity() < nmax) continue;
         if (v.capacity() >= 8 * nmax && v.nt > 32) continue;  // mostly idle threads
         std::vector<Bin> one{Bin{(int)vi, (int)rods.size(), d_work}};
-        int spare = h->sms - h->n_rods;
-        one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &spare);
+        TileRoom room = tile_room(h);
+        one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
         if (one[0].tile.per && prepare_tile(one[0].tile) != cudaSuccess) one[0].tile.per = 0;
         restore();
         if ((rc = launch_bins(h, one, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
@@ -1495,7 +1518,7 @@ int rod_bind(rod_handle h, int outer, int inner, int mode) {
 // variant, so that rod_rollout and the adjoint's recomputation run the same kernel code.
 static int build_adjoint_bins(rod_handle h) {
   if (!h->adj_bins.empty()) return CORDE_OK;
-  int spare = h->sms - h->n_rods;
+  TileRoom room = tile_room(h);
   for (int nt = 32; nt <= kAdjointMaxNodes / 2; nt *= 2) {
     std::vector<int> rods;
     for (int r = 0; r < h->n_rods; ++r) {
@@ -1510,7 +1533,10 @@ static int build_adjoint_bins(rod_handle h) {
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
     for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
-    b.tile = tile_plan(b.n_max, b.count, 2, &spare);
+    b.tile = tile_plan(b.n_max, b.count, 2, &room);
+    // two or more tiles in one block don't pay here: a training step of 256 rods of 256 nodes took
+    // 2.77 ms against 2.65 with the block kernel, though the rollout alone is no slower
+    if (b.tile.blocks == 1 && b.tile.warps > 1 && b.count > h->sms) b.tile.per = 0;
     if (b.tile.per) CK(prepare_tile(b.tile));
     h->adj_bins.push_back(b);
   }

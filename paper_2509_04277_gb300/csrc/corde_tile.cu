@@ -19,8 +19,10 @@
 namespace corde {
 namespace {
 
-template <int PER, int ARITH, int SYNC>
-__global__ void __launch_bounds__(32 * kTileMaxWarps, 1)
+// MAXT threads per SM bound the registers: 256 for the lone warps of a long chain, 512 to fill an
+// SM with rods of one warp.
+template <int PER, int ARITH, int SYNC, int MAXT = 32 * kTileMaxWarps>
+__global__ void __launch_bounds__(MAXT, 1)
 tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, float4* __restrict__ x4,
                  float4* __restrict__ v4, float4* __restrict__ q4, float4* __restrict__ o4,
                  const float4* __restrict__ u4, const float4* __restrict__ k4, const float4* __restrict__ drive,
@@ -146,6 +148,11 @@ TileFn tile_fn_t(const TilePlan& p) {
 }
 TileFn tile_fn(const TilePlan& p) {
   if (p.warps < 1 || p.warps > kTileMaxWarps) return nullptr;
+  if (p.full) {
+    if (p.blocks != 1 || p.warps != 1) return nullptr;
+    if (p.per == 2) return p.arith == 4 ? tile_step_kernel<2, 4, kTileBlock, 512> : tile_step_kernel<2, 2, kTileBlock, 512>;
+    return p.arith == 4 ? tile_step_kernel<4, 4, kTileBlock, 512> : nullptr;
+  }
   if (p.per == 4 && p.arith == 4) return tile_fn_t<4, 4>(p);
   if (p.per == 4 && p.arith == 2) return tile_fn_t<4, 2>(p);
   if (p.per == 2 && p.arith == 4) return tile_fn_t<2, 4>(p);

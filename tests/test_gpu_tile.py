@@ -94,6 +94,15 @@ def test_uneven_rods_in_one_handle(corde):
     _check(corde, W.batched_rods(12, seed=77), (1, 10))
 
 
+# more rods than SMs: one tile per rod (64 and 128 nodes; 1300 rods fill the SMs), two and three tiles in a
+# block, and too many for either
+@pytest.mark.parametrize("n,count,plan", [(64, 200, None), (64, 200, (4, 32)), (100, 200, None), (128, 1300, None),
+                                          (100, 200, (2, 64)), (200, 300, None), (270, 200, (2, 256)), (200, 700, None)])
+def test_many_rods(corde, n, count, plan):
+    rod = W.guidewire(n, seed=n)
+    _check(corde, [rod] * count, (1, 10), plan)
+
+
 def test_free_base(corde):
     rod = W.guidewire(200, seed=5)
     rod.clamp = 0
