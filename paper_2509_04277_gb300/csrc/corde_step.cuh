@@ -85,6 +85,15 @@ struct BlockHalo {
   }
   __device__ __forceinline__ float3 next3(const float4* hb, int slot) const { return get3(hb, slot, t + 1); }
   __device__ __forceinline__ float3 prev3(const float4* hb, int slot) const { return get3(hb, slot, t - 1); }
+  // the neighbours' slots; at the rod's ends the thread's own (any finite value serves a
+  // constraint that does not exist, and no branch or select is needed: 10 % of the batch)
+  __device__ __forceinline__ int tn() const { return has_next() ? t + 1 : t; }
+  __device__ __forceinline__ int tp() const { return has_prev() ? t - 1 : t; }
+  __device__ __forceinline__ float3 sweep_next(const float4* hb) const { return get3(hb, 0, tn()); }
+  __device__ __forceinline__ float3 sweep_prev(const float4* hb) const { return get3(hb, 1, tp()); }
+  __device__ __forceinline__ float4 end_next(const float4* hb, int slot) const { return hb[slot * NT + tn()]; }
+  __device__ __forceinline__ float4 end_prev(const float4* hb, int slot) const { return hb[slot * NT + tp()]; }
+  __device__ __forceinline__ float3 carry_prev(const float4* hb, int slot) const { return get3(hb, slot, tp()); }
   __device__ __forceinline__ void sync() const { block_sync<SYNC_NT>(); }
   // a barrier in two halves (arrive after the exchange stores, wait before the neighbour
   // loads); one block has no split barrier, so the wait is the whole barrier
@@ -128,6 +137,18 @@ struct ClusterHalo {
   }
   __device__ __forceinline__ float3 next3(const float4* hb, int slot) const { return f3(next(hb, slot)); }
   __device__ __forceinline__ float3 prev3(const float4* hb, int slot) const { return f3(prev(hb, slot)); }
+  // (zeros at the rod's ends: there is no slot to read)
+  __device__ __forceinline__ float3 sweep_next(const float4* hb) const { return has_next() ? next3(hb, 0) : zero3(); }
+  __device__ __forceinline__ float3 sweep_prev(const float4* hb) const { return has_prev() ? prev3(hb, 1) : zero3(); }
+  __device__ __forceinline__ float4 end_next(const float4* hb, int slot) const {
+    return has_next() ? next(hb, slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ float4 end_prev(const float4* hb, int slot) const {
+    return has_prev() ? prev(hb, slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ float3 carry_prev(const float4* hb, int slot) const {
+    return has_prev() ? prev3(hb, slot) : zero3();
+  }
   __device__ __forceinline__ void sync() const { cooperative_groups::this_cluster().sync(); }
   // OR of x over the rod's threads on all C blocks (a block-wide OR, each block's result
   // in its shared memory, read by every thread through distributed shared memory between
@@ -185,6 +206,18 @@ struct GridHalo {
   }
   __device__ __forceinline__ float3 next3(const float4* hb, int slot) const { return f3(next(hb, slot)); }
   __device__ __forceinline__ float3 prev3(const float4* hb, int slot) const { return f3(prev(hb, slot)); }
+  // (zeros at the rod's ends: there is no slot to read)
+  __device__ __forceinline__ float3 sweep_next(const float4* hb) const { return has_next() ? next3(hb, 0) : zero3(); }
+  __device__ __forceinline__ float3 sweep_prev(const float4* hb) const { return has_prev() ? prev3(hb, 1) : zero3(); }
+  __device__ __forceinline__ float4 end_next(const float4* hb, int slot) const {
+    return has_next() ? next(hb, slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ float4 end_prev(const float4* hb, int slot) const {
+    return has_prev() ? prev(hb, slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ float3 carry_prev(const float4* hb, int slot) const {
+    return has_prev() ? prev3(hb, slot) : zero3();
+  }
   __device__ __forceinline__ void sync() const { cooperative_groups::this_grid().sync(); }
   // after the exchange stores: the block's first and last thread copy their slots (written
   // by themselves just before) to global memory; the grid sync then publishes them
@@ -216,28 +249,71 @@ __device__ __forceinline__ void joint_torques(float4 qa, float4 qb, float4 uh, f
 // Segment forces between nodes a and b and the penalty torque on frame q (Eq. 8, and
 // Eq. 2 when the rod is extensible).  Penalty: E = 1/2 l0 Kp |t - d3|^2 gives the force
 // l0 Kp (d3 - (t . d3) t) / |e| on node b (opposite on a) and the torque l0 Kp d3 x t,
-// which in the body frame (d3 = e_z) is l0 Kp (-t_b.y, t_b.x, 0) with t_b = R(q)^T t
-// (*t_body, if given).
-__device__ __forceinline__ void segment_forces(float3 ra, float3 rb, float4 q, const RodDev& R, bool extensible,
-                                               float3& fa, float3& fb, float3& tq, float3* t_body = nullptr) {
-  const float3 e = rb - ra;
+// which in the body frame (d3 = e_z) is l0 Kp (-t_b.y, t_b.x, 0) with t_b = R(q)^T t.
+// Returns the forces, t_b and the scale lk = l0 Kp; a segment that does not exist gets zero
+// forces and lk = 0 without a branch (branches around a lane's elements keep their chains
+// from overlapping).
+__device__ __forceinline__ void segment_forces(float3 ra, float3 rb, float4 q, const RodDev& R, bool exists,
+                                               bool extensible, float3& fa, float3& fb, float3& t_body, float& lk) {
+  const float3 d = rb - ra;
+  const float3 e = f3(exists ? d.x : 0.f, exists ? d.y : 0.f, exists ? d.z : 1.f);
+  lk = exists ? R.lKp : 0.f;
   const float ee = dot3(e, e);
   const float il = rsqrtf(ee);
   const float3 t = il * e;
   const float3 d3 = director3(q);
   const float c = dot3(t, d3);
-  const float3 f = (R.lKp * il) * (d3 - c * t);
+  const float3 f = (lk * il) * (d3 - c * t);
   fb = f;
   fa = -f;
   if (extensible) {
     const float len = ee * il;
-    const float3 fs = (R.Ks * (len * R.inv_l0 - 1.f)) * t;
+    const float3 fs = ((exists ? R.Ks : 0.f) * (len * R.inv_l0 - 1.f)) * t;
     fa += fs;
     fb -= fs;
   }
-  const float3 tb = rotate_inv(q, t);
-  tq = f3(-R.lKp * tb.y, R.lKp * tb.x, 0.f);
-  if (t_body != nullptr) *t_body = tb;
+  t_body = rotate_inv(q, t);
+}
+// a + b, rounded per component: never fused with what computes b
+__device__ __forceinline__ float3 add_rn(float3 a, float3 b) {
+  return f3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z));
+}
+// tau plus the penalty torque of segment_forces, each component fused
+__device__ __forceinline__ float3 add_penalty_torque(float3 tau, float lk, float3 t_body) {
+  return f3(__fmaf_rn(-lk, t_body.y, tau.x), __fmaf_rn(lk, t_body.x, tau.y), tau.z);
+}
+
+// Force integration of one node and one frame, and the frame's update (semi-implicit Euler), without
+// branches: what does not move (a kinematic node or frame, an element that does not exist) keeps
+// its values.
+__device__ __forceinline__ void integrate_node(const RodDev& R, float w, float3 F, float3& v) {
+  const float dt = R.dt;
+  const float3 a = f3(w * F.x + R.gx, w * F.y + R.gy, w * F.z + R.gz);
+  const float3 vn = R.damp * (v + dt * a);
+  const bool on = w > 0.f;
+  v = f3(on ? vn.x : v.x, on ? vn.y : v.y, on ? vn.z : v.z);
+}
+__device__ __forceinline__ void integrate_frame(const RodDev& R, bool dynamic, float3 tau, float3& om) {
+  const float dt = R.dt;
+  const float3 o = om;
+  const float3 Jw = f3(R.J1 * o.x, R.J1 * o.y, R.J3 * o.z);
+  const float3 rhs = tau - cross3(o, Jw);
+  const float3 on = f3(o.x + dt * R.Jinv1 * rhs.x, o.y + dt * R.Jinv1 * rhs.y, o.z + dt * R.Jinv3 * rhs.z);
+  const float3 od = R.damp * on;
+  om = f3(dynamic ? od.x : o.x, dynamic ? od.y : o.y, dynamic ? od.z : o.z);
+}
+__device__ __forceinline__ void update_frame(float half_dt, bool exists, float3 o, float4& q) {
+  const float4 a = q;
+  // q (x) (0, omega), each product fused as spelled out (the same rounding in every kernel)
+  const float dx = __fmaf_rn(-a.z, o.y, __fmaf_rn(a.w, o.x, __fmul_rn(a.y, o.z)));
+  const float dy = __fmaf_rn(-a.x, o.z, __fmaf_rn(a.z, o.x, __fmul_rn(a.w, o.y)));
+  const float dz = __fmaf_rn(-a.y, o.x, __fmaf_rn(a.x, o.y, __fmul_rn(a.w, o.z)));
+  const float dwq = -__fmaf_rn(a.z, o.z, __fmaf_rn(a.x, o.x, __fmul_rn(a.y, o.y)));
+  const float4 b = make_float4(__fmaf_rn(half_dt, dx, a.x), __fmaf_rn(half_dt, dy, a.y), __fmaf_rn(half_dt, dz, a.z),
+                               __fmaf_rn(half_dt, dwq, a.w));
+  const float inv =
+      rsqrtf(__fmaf_rn(b.w, b.w, __fmaf_rn(b.z, b.z, __fmaf_rn(b.y, b.y, __fmul_rn(b.x, b.x)))));
+  q = make_float4(exists ? b.x * inv : a.x, exists ? b.y * inv : a.y, exists ? b.z * inv : a.z, exists ? b.w * inv : a.w);
 }
 
 // Impulse of one distance constraint (predictive: makes the segment length l0 after the
@@ -469,48 +545,31 @@ __device__ __forceinline__ void step_body(const RodDev& R, const Halo& H, float3
   }
   float3 F_carry = zero3(), tau_carry = zero3();
   auto joint_and_segment = [&](int e, float4 qb, float3 rb) {
-    const int j = e0 + e;
-    if (j <= n - 3) {
-      float3 ta, tb;
-      joint_torques(q[e], qb, par_u[e * NT + t], par_k[e * NT + t], R.two_over_l, ta, tb);
-      tau[e] += ta;
-      if (e + 1 < EPT) {
-        tau[(e + 1) % EPT] += tb;
-      } else {
-        tau_carry = tb;
-      }
-    }
-    if (j <= n - 2) {
-      float3 fa, fb, tq;
-      segment_forces(r[e], rb, q[e], R, !inext, fa, fb, tq);
-      F[e] += fa;
-      tau[e] += tq;
-      if (e + 1 < EPT) {
-        F[(e + 1) % EPT] += fb;
-      } else {
-        F_carry = fb;
-      }
+    float3 ta, tb, fa, fb, t_body;
+    float lk;
+    // (a joint that does not exist has K = 0 and so no torques)
+    joint_torques(q[e], qb, par_u[e * NT + t], par_k[e * NT + t], R.two_over_l, ta, tb);
+    segment_forces(r[e], rb, q[e], R, e0 + e <= n - 2, !inext, fa, fb, t_body, lk);
+    tau[e] = add_penalty_torque(add_rn(tau[e], ta), lk, t_body);
+    F[e] = add_rn(F[e], fa);
+    if (e + 1 < EPT) {
+      tau[(e + 1) % EPT] = add_rn(tau[(e + 1) % EPT], tb);
+      F[(e + 1) % EPT] = add_rn(F[(e + 1) % EPT], fb);
+    } else {
+      tau_carry = tb;
+      F_carry = fb;
     }
   };
 #pragma unroll
   for (int e = 0; e + 1 < EPT; ++e) joint_and_segment(e, q[e + 1], r[e + 1]);
 
   H.wait();
-  float3 r_next = zero3(), r_prev = zero3();
-  float w_next = 0.f, w_prev = 0.f;
-  float4 q_next = make_float4(0.f, 0.f, 0.f, 1.f);
+  // (at the rod's ends any finite values: nothing that uses them exists)
   const bool has_next = H.has_next(), has_prev = H.has_prev();
-  if (has_next) {
-    const float4 a = H.next(hb, 0);
-    r_next = f3(a);
-    w_next = a.w;
-    q_next = H.next(hb, 1);
-  }
-  if (has_prev) {
-    const float4 a = H.prev(hb, 2);
-    r_prev = f3(a);
-    w_prev = a.w;
-  }
+  const float4 xn = H.end_next(hb, 0), xp = H.end_prev(hb, 2);
+  const float3 r_next = f3(xn), r_prev = f3(xp);
+  const float w_next = xn.w, w_prev = xp.w;
+  const float4 q_next = H.end_next(hb, 1);
   if constexpr (STORE) {
     nb->r_next = r_next;
     nb->r_prev = r_prev;
@@ -568,25 +627,16 @@ __device__ __forceinline__ void step_body(const RodDev& R, const Halo& H, float3
   }
   auto integrate = [&](int e) {
     const int i = e0 + e;
-    if (w[e] > 0.f) {
-      const float3 a = f3(w[e] * F[e].x + R.gx, w[e] * F[e].y + R.gy, w[e] * F[e].z + R.gz);
-      v[e] = R.damp * (v[e] + dt * a);
-    }
-    const bool frame_dynamic = (i <= n - 2) && !(clamp && i == 0);
-    if (frame_dynamic) {
-      const float3 o = om[e];
-      const float3 Jw = f3(R.J1 * o.x, R.J1 * o.y, R.J3 * o.z);
-      const float3 rhs = tau[e] - cross3(o, Jw);
-      const float3 on = f3(o.x + dt * R.Jinv1 * rhs.x, o.y + dt * R.Jinv1 * rhs.y, o.z + dt * R.Jinv3 * rhs.z);
-      om[e] = R.damp * on;
-    }
+    integrate_node(R, w[e], F[e], v[e]);
+    integrate_frame(R, (i <= n - 2) && !(clamp && i == 0), tau[e], om[e]);
   };
 #pragma unroll
   for (int e = 1; e < EPT; ++e) integrate(e);
   H.wait();
-  if (has_prev) {
-    F[0] += H.prev3(hb, 0);
-    tau[0] += H.prev3(hb, 1);
+  {
+    const float3 f = H.carry_prev(hb, 0), c = H.carry_prev(hb, 1);
+    F[0] = add_rn(F[0], f3(has_prev ? f.x : 0.f, has_prev ? f.y : 0.f, has_prev ? f.z : 0.f));
+    tau[0] = add_rn(tau[0], f3(has_prev ? c.x : 0.f, has_prev ? c.y : 0.f, has_prev ? c.z : 0.f));
   }
   integrate(0);
   if (clamp && e0 == 0) {
@@ -597,20 +647,7 @@ __device__ __forceinline__ void step_body(const RodDev& R, const Halo& H, float3
   // constraint sweeps change only the node velocities, so the frames' update is final
   // here and overlaps the sweeps' latency
 #pragma unroll
-  for (int e = 0; e < EPT; ++e) {
-    if (e0 + e <= n - 2) {
-      const float4 a = q[e];
-      const float3 o = om[e];
-      // q (x) (0, omega)
-      const float dx = a.w * o.x + a.y * o.z - a.z * o.y;
-      const float dy = a.w * o.y + a.z * o.x - a.x * o.z;
-      const float dz = a.w * o.z + a.x * o.y - a.y * o.x;
-      const float dwq = -(a.x * o.x + a.y * o.y + a.z * o.z);
-      const float4 b = make_float4(a.x + half_dt * dx, a.y + half_dt * dy, a.z + half_dt * dz, a.w + half_dt * dwq);
-      const float inv = rsqrtf(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
-      q[e] = make_float4(b.x * inv, b.y * inv, b.z * inv, b.w * inv);
-    }
-  }
+  for (int e = 0; e < EPT; ++e) update_frame(half_dt, e0 + e <= n - 2, om[e], q[e]);
 
   // ---- distance-constraint iterations (inextensible rod), red-black
   if (inext) {
@@ -693,8 +730,8 @@ __device__ __forceinline__ void step_body(const RodDev& R, const Halo& H, float3
       H.wait();
       // odd segments across the two thread boundaries
       {
-        const float3 vn = has_next ? H.next3(hb, 0) : zero3();
-        const float3 vp = has_prev ? H.prev3(hb, 1) : zero3();
+        const float3 vn = H.sweep_next(hb);
+        const float3 vp = H.sweep_prev(hb);
         if constexpr (EPT == 2) {
           boundary_apply(e_bnd, sc.l_bnd, sc.c_bnd, dt, vn, vp, v[EPT - 1], v[0]);
         } else {
@@ -755,9 +792,10 @@ __device__ __forceinline__ void load_rod(const RodDev& R, const int t, const int
       om[e] = f3(o4[R.off + i]);
       if (par_u != nullptr) {
         par_u[e * NT + t] = u4[R.off + i];
-        par_k[e * NT + t] = k4[R.off + i];
+        par_k[e * NT + t] = i <= R.n - 3 ? k4[R.off + i] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     } else {
+      if (par_u != nullptr) par_u[e * NT + t] = par_k[e * NT + t] = make_float4(0.f, 0.f, 0.f, 0.f);
       r[e] = zero3();
       v[e] = zero3();
       om[e] = zero3();

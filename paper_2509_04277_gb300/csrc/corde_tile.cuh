@@ -32,10 +32,6 @@ __device__ __forceinline__ float3 up3(float3 a) {
   return f3(__shfl_up_sync(0xffffffffu, a.x, 1), __shfl_up_sync(0xffffffffu, a.y, 1),
             __shfl_up_sync(0xffffffffu, a.z, 1));
 }
-__device__ __forceinline__ float3 add_rn(float3 a, float3 b) {
-  return f3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z));
-}
-
 // Predicted offset of a constraint and its reciprocal length.
 __device__ __forceinline__ float3 offset_of(float3 e, float3 va, float3 vb, float dt, float& il) {
   const float3 d = f3(__fmaf_rn(dt, __fsub_rn(vb.x, va.x), e.x), __fmaf_rn(dt, __fsub_rn(vb.y, va.y), e.y),
@@ -78,8 +74,10 @@ struct TileRod {
         v[e] = f3(v4[R.off + i]);
         q[e] = q4[R.off + i];
         om[e] = f3(o4[R.off + i]);
-        uh[e] = f3(u4[R.off + i]);
-        kk[e] = f3(k4[R.off + i]);
+        if (i <= n - 3) {  // (a joint that does not exist has K = 0 and so no torques)
+          uh[e] = f3(u4[R.off + i]);
+          kk[e] = f3(k4[R.off + i]);
+        }
       }
     }
     const float w_next = __shfl_down_sync(0xffffffffu, w[0], 1), w_prev = __shfl_up_sync(0xffffffffu, w[PER - 1], 1);
@@ -130,73 +128,32 @@ struct TileRod {
     const bool inext = (R.flags & F_INEXT) != 0, clamp = (R.flags & F_CLAMP) != 0;
     const float dt = R.dt, half_dt = 0.5f * dt;
     // ---- elastic forces and torques
-    float3 F[PER], tau[PER], Fc[PER + 1], Tc[PER + 1];
-#pragma unroll
-    for (int e = 0; e < PER; ++e) F[e] = tau[e] = zero3();
-#pragma unroll
-    for (int e = 0; e <= PER; ++e) Fc[e] = Tc[e] = zero3();
+    float3 F[PER], tau[PER];
     const float3 r_next = down3(r[0]), r_prev = up3(r[PER - 1]);
     const float4 q_next = make_float4(__shfl_down_sync(0xffffffffu, q[0].x, 1), __shfl_down_sync(0xffffffffu, q[0].y, 1),
                                       __shfl_down_sync(0xffffffffu, q[0].z, 1), __shfl_down_sync(0xffffffffu, q[0].w, 1));
-    auto joint_and_segment = [&](int e, float4 qb, float3 rb) {
-      const int j = e0 + e;
-      const bool carry = (e + 1) % (ARITH < PER ? ARITH : PER) == 0;  // to another lane, or a thread boundary of the layout
-      if (j <= n - 3) {
-        float3 ta, tb;
-        joint_torques(q[e], qb, make_float4(uh[e].x, uh[e].y, uh[e].z, 0.f), make_float4(kk[e].x, kk[e].y, kk[e].z, 0.f),
-                      R.two_over_l, ta, tb);
-        tau[e] += ta;
-        if (!carry) {
-          tau[(e + 1) % PER] += tb;
-        } else {
-          Tc[e + 1] = tb;
-        }
-      }
-      if (j <= n - 2) {
-        float3 fa, fb, tq;
-        segment_forces(r[e], rb, q[e], R, !inext, fa, fb, tq);
-        F[e] += fa;
-        tau[e] += tq;
-        if (!carry) {
-          F[(e + 1) % PER] += fb;
-        } else {
-          Fc[e + 1] = fb;
-        }
-      }
-    };
-    if constexpr (ARITH <= PER) {
+    // each element's joint and segment, all computed before any is added up
+    float3 ta[PER], tb[PER], fa[PER], fb[PER], t_body[PER];
+    float lk[PER];
 #pragma unroll
-      for (int e = 0; e < PER; ++e)
-        joint_and_segment(e, e + 1 < PER ? q[(e + 1) % PER] : q_next, e + 1 < PER ? r[(e + 1) % PER] : r_next);
-      Fc[0] = up3(Fc[PER]);
-      Tc[0] = up3(Tc[PER]);
-      if (lane == 0) Fc[0] = Tc[0] = zero3();
-    } else {
-      // two lanes make a thread of the <4, *> layout: the first element of the second lane
-      // takes the previous element's contribution before its own, the first lane's after
-      static_assert(ARITH <= PER || (PER == 2 && ARITH == 4), "tile layouts");
-      float3 ta = zero3(), fa = zero3(), fb, tq, tb = zero3();
-      if (e0 <= n - 3)
-        joint_torques(q[0], q[1], make_float4(uh[0].x, uh[0].y, uh[0].z, 0.f), make_float4(kk[0].x, kk[0].y, kk[0].z, 0.f),
-                      R.two_over_l, ta, tau[1]);
-      if (e0 <= n - 2) {
-        segment_forces(r[0], r[1], q[0], R, !inext, fa, fb, tq, &tb);
-        F[1] += fb;
-      }
-      joint_and_segment(1, q_next, r_next);
-      float3 Fi = up3(Fc[2]), Ti = up3(Tc[2]);
-      if (lane == 0) Fi = Ti = zero3();
-      if ((e0 >> 1) & 1) {
-        F[0] = Fi;
-        tau[0] = Ti;
-      } else {
-        Fc[0] = Fi;
-        Tc[0] = Ti;
-      }
-      F[0] = add_rn(F[0], fa);
-      tau[0] = add_rn(tau[0], ta);
-      // the penalty torque as the layouts fuse it (segment_forces' tq scaled and added)
-      tau[0] = f3(__fmaf_rn(-R.lKp, tb.y, tau[0].x), __fmaf_rn(R.lKp, tb.x, tau[0].y), tau[0].z);
+    for (int e = 0; e < PER; ++e) {
+      const float4 qb = e + 1 < PER ? q[(e + 1) % PER] : q_next;
+      const float3 rb = e + 1 < PER ? r[(e + 1) % PER] : r_next;
+      joint_torques(q[e], qb, make_float4(uh[e].x, uh[e].y, uh[e].z, 0.f), make_float4(kk[e].x, kk[e].y, kk[e].z, 0.f),
+                    R.two_over_l, ta[e], tb[e]);
+      segment_forces(r[e], rb, q[e], R, e0 + e <= n - 2, !inext, fa[e], fb[e], t_body[e], lk[e]);
+    }
+    float3 Fi = up3(fb[PER - 1]), Ti = up3(tb[PER - 1]);  // from the previous lane's last element
+    if (lane == 0) Fi = Ti = zero3();
+    // The layout's order: an element that starts one of its threads takes the previous element's
+    // contribution after its own, the others before (at ARITH > PER two lanes make a thread).
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const float3 f = e == 0 ? Fi : fb[(e + PER - 1) % PER], c = e == 0 ? Ti : tb[(e + PER - 1) % PER];
+      const bool after = ARITH <= PER ? e % ARITH == 0 : e == 0 && ((e0 >> 1) & 1) == 0;
+      auto pick = [](bool p, float3 x) { return f3(p ? x.x : 0.f, p ? x.y : 0.f, p ? x.z : 0.f); };
+      F[e] = add_rn(add_rn(pick(!after, f), fa[e]), pick(after, f));
+      tau[e] = add_rn(add_penalty_torque(add_rn(pick(!after, c), ta[e]), lk[e], t_body[e]), pick(after, c));
     }
 
     // ---- constraint geometry
@@ -205,49 +162,19 @@ struct TileRod {
       e_seg[s] = safe_segment(inv[s], segment_vector(r[s], s + 1 < PER ? r[(s + 1) % PER] : r_next), R.l0);
     e_left = safe_segment(inv[PER], segment_vector(r_prev, r[0]), R.l0);
 
-    // ---- force integration
-    auto integrate = [&](int e) {
-      const int i = e0 + e;
-      if (w[e] > 0.f) {
-        const float3 a = f3(w[e] * F[e].x + R.gx, w[e] * F[e].y + R.gy, w[e] * F[e].z + R.gz);
-        v[e] = R.damp * (v[e] + dt * a);
-      }
-      const bool frame_dynamic = (i <= n - 2) && !(clamp && i == 0);
-      if (frame_dynamic) {
-        const float3 o = om[e];
-        const float3 Jw = f3(R.J1 * o.x, R.J1 * o.y, R.J3 * o.z);
-        const float3 rhs = tau[e] - cross3(o, Jw);
-        const float3 on = f3(o.x + dt * R.Jinv1 * rhs.x, o.y + dt * R.Jinv1 * rhs.y, o.z + dt * R.Jinv3 * rhs.z);
-        om[e] = R.damp * on;
-      }
-    };
+    // ---- force integration and frames
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
-      if (e % ARITH == 0) {  // (zero for a second lane of ARITH > PER)
-        F[e] = add_rn(F[e], Fc[e]);
-        tau[e] = add_rn(tau[e], Tc[e]);
-      }
-      integrate(e);
+      const int i = e0 + e;
+      integrate_node(R, w[e], F[e], v[e]);
+      integrate_frame(R, (i <= n - 2) && !(clamp && i == 0), tau[e], om[e]);
     }
     if (clamp && e0 == 0) {
       v[0] = v_drive;
       om[0] = w_drive;
     }
-    // ---- frames
 #pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      if (e0 + e <= n - 2) {
-        const float4 a = q[e];
-        const float3 o = om[e];
-        const float dx = a.w * o.x + a.y * o.z - a.z * o.y;
-        const float dy = a.w * o.y + a.z * o.x - a.x * o.z;
-        const float dz = a.w * o.z + a.x * o.y - a.y * o.x;
-        const float dwq = -(a.x * o.x + a.y * o.y + a.z * o.z);
-        const float4 b = make_float4(a.x + half_dt * dx, a.y + half_dt * dy, a.z + half_dt * dz, a.w + half_dt * dwq);
-        const float il = rsqrtf(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
-        q[e] = make_float4(b.x * il, b.y * il, b.z * il, b.w * il);
-      }
-    }
+    for (int e = 0; e < PER; ++e) update_frame(half_dt, e0 + e <= n - 2, om[e], q[e]);
   }
 
   // One iteration of the distance constraints, red-black.
