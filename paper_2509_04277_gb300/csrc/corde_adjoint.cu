@@ -51,8 +51,8 @@ struct BlockNet {
     H.put3(hb, 0, first);
     H.put3(hb, 1, last);
     block_sync<NT>();
-    next = H.next3(hb, 0);
-    prev = H.prev3(hb, 1);
+    next = H.sweep_next(hb);
+    prev = H.sweep_prev(hb);
   }
   // the next thread's a and b
   __device__ __forceinline__ void swap_forces(float3 a, float3 b, float3& an, float3& bn) {

@@ -44,7 +44,9 @@ __global__ void __launch_bounds__(32 * kTileMaxWarps, 1) tile_record_kernel(Adjo
     v_drive = f3(a.drive[2 * rid]);
     w_drive = f3(a.drive[2 * rid + 1]);
   }
-  const bool keeps = link.owned && rod.e0 < rod.n;
+  // lanes beyond the rod's end write their zeros too: the reverse pass reads whole windows, and an
+  // absent constraint times zero has to be zero
+  const bool keeps = link.owned;
   const int t0 = seg * a.ckpt_every, cnt = min(a.ckpt_every, a.n_steps - t0);
   const int n_iters = (R.flags & F_INEXT) ? R.n_iters : 0;
   auto put_state = [&](int step) {

@@ -217,7 +217,7 @@ pair_kernel(const RodDev* __restrict__ rods, const int4* __restrict__ pairs, flo
     if (i < R.n) {
       x4[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
       v4[R.off + i] = make_float4(v[e].x, v[e].y, v[e].z, 0.f);
-      q4[R.off + i] = q[e];
+      if (i <= R.n - 2) q4[R.off + i] = q[e];
       o4[R.off + i] = make_float4(om[e].x, om[e].y, om[e].z, 0.f);
       if (pos_out != nullptr) pos_out[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
     }

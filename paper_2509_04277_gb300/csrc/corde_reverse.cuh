@@ -114,8 +114,8 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // the caller applies va_bar -= dt d_bar, vb_bar += dt d_bar, ra_bar -= d_bar, rb_bar += d_bar.
 // In two parts: the geometry (direction n and l0/L of the predicted segment) depends only
 // on the recorded velocities, so it is computed before the exchange of the adjoint velocities;
-// inv = -1/(dt W) is constant over a step, and 0 for a constraint that does not exist (its
-// geometry is then a safe unit vector and the returned d_bar is 0).
+// inv = -1/(dt W) is constant over a step, and 0 for a constraint that does not exist (the
+// returned d_bar is then 0).
 struct VjpGeo {
   float3 n;
   float rho;
@@ -123,15 +123,17 @@ struct VjpGeo {
 __device__ __forceinline__ float vjp_inv(bool exists, float wa, float wb, float dt) {
   return (exists && wa + wb > 0.f) ? -__frcp_rn(__fmul_rn(dt, wa + wb)) : 0.f;
 }
-__device__ __forceinline__ VjpGeo vjp_geo(float3 ra, float3 va, float3 rb, float3 vb, float inv, float l0,
-                                          float dt) {
-  float3 d = f3(__fmaf_rn(dt, __fsub_rn(vb.x, va.x), __fsub_rn(rb.x, ra.x)),
-                __fmaf_rn(dt, __fsub_rn(vb.y, va.y), __fsub_rn(rb.y, ra.y)),
-                __fmaf_rn(dt, __fsub_rn(vb.z, va.z), __fsub_rn(rb.z, ra.z)));
-  if (inv == 0.f) d = f3(0.f, 0.f, 1.f);
+// e = r_b - r_a, a safe vector where the constraint does not exist (see vjp_segment)
+__device__ __forceinline__ VjpGeo vjp_geo(float3 e, float3 va, float3 vb, float l0, float dt) {
+  const float3 d = f3(__fmaf_rn(dt, __fsub_rn(vb.x, va.x), e.x), __fmaf_rn(dt, __fsub_rn(vb.y, va.y), e.y),
+                      __fmaf_rn(dt, __fsub_rn(vb.z, va.z), e.z));
   const float dd = __fmaf_rn(d.x, d.x, __fmaf_rn(d.y, d.y, __fmul_rn(d.z, d.z)));
   const float il = rsqrtf(dd);
   return VjpGeo{il * d, l0 * il};
+}
+// The safe vector is long against any dt v, so that the predicted segment cannot vanish.
+__device__ __forceinline__ float3 vjp_segment(float inv, float3 ra, float3 rb) {
+  return inv != 0.f ? segment_vector(ra, rb) : f3(0.f, 0.f, 1e6f);
 }
 __device__ __forceinline__ float3 vjp_apply(const VjpGeo& G, float inv, float wa, float wb, float3 va_bar,
                                             float3 vb_bar) {
@@ -191,7 +193,10 @@ __device__ __forceinline__ void reverse_step(const RodDev& R, Net& net, const fl
     const float inv_e = vjp_inv(e0 + 1 <= n - 1, w[0], w[1], dt);
     const float inv_r = vjp_inv(net.has_next() && e0 + EPT <= n - 1, w[EPT - 1], nb.w_next, dt);
     const float inv_l = Net::kShared ? 0.f : vjp_inv(net.has_prev() && e0 <= n - 1, nb.w_prev, w[0], dt);
-    // the forward's boundary segment vectors (positions are fixed during the sweeps)
+    // the segment vectors (positions are fixed during the sweeps), once per step
+    const float3 s_r = vjp_segment(inv_r, r[EPT - 1], nb.r_next), s_e = vjp_segment(inv_e, r[0], r[1]);
+    const float3 s_l = Net::kShared ? zero3() : vjp_segment(inv_l, nb.r_prev, r[0]);
+    // the forward's boundary segment vectors
     const float3 e_r = safe_segment(sc.i_right, segment_vector(r[EPT - 1], nb.r_next), R.l0);
     const float3 e_l = safe_segment(sc.i_left, segment_vector(nb.r_prev, r[0]), R.l0);
     const Vec3x2 e_bnd{make_float2(e_r.x, e_l.x), make_float2(e_r.y, e_l.y), make_float2(e_r.z, e_l.z)};
@@ -217,21 +222,21 @@ __device__ __forceinline__ void reverse_step(const RodDev& R, Net& net, const fl
           }
         }
       }
-      const VjpGeo g_r = vjp_geo(r[EPT - 1], net.rec(so, EPT - 1), nb.r_next, net.rec_next(so), inv_r, R.l0, dt);
+      const VjpGeo g_r = vjp_geo(s_r, net.rec(so, EPT - 1), net.rec_next(so), R.l0, dt);
       VjpGeo g_l;
-      if constexpr (!Net::kShared) g_l = vjp_geo(nb.r_prev, net.rec_prev(so), r[0], net.rec(so, 0), inv_l, R.l0, dt);
-      const VjpGeo g_e = vjp_geo(r[0], ve[0], r[1], ve[1], inv_e, R.l0, dt);
+      if constexpr (!Net::kShared) g_l = vjp_geo(s_l, net.rec_prev(so), net.rec(so, 0), R.l0, dt);
+      const VjpGeo g_e = vjp_geo(s_e, ve[0], ve[1], R.l0, dt);
       // exchange of the adjoint velocities of the first and last element
-      float3 vn_bar, vp_bar;  // meaningful only where the constraint exists
+      float3 vn_bar, vp_bar;  // (finite where there is no neighbour)
       net.swap_velocities(vb2[0], vb2[EPT - 1], vn_bar, vp_bar);
-      const float3 db_r = vjp_apply(g_r, inv_r, w[EPT - 1], nb.w_next, vb2[EPT - 1], net.has_next() ? vn_bar : zero3());
+      const float3 db_r = vjp_apply(g_r, inv_r, w[EPT - 1], nb.w_next, vb2[EPT - 1], vn_bar);
       vb2[EPT - 1] -= dt * db_r;
       rb[EPT - 1] -= db_r;
       float3 db_l;
       if constexpr (Net::kShared) {
         db_l = net.from_prev(db_r);
       } else {
-        db_l = vjp_apply(g_l, inv_l, nb.w_prev, w[0], net.has_prev() ? vp_bar : zero3(), vb2[0]);
+        db_l = vjp_apply(g_l, inv_l, nb.w_prev, w[0], vp_bar, vb2[0]);
       }
       vb2[0] += dt * db_l;
       rb[0] += db_l;

@@ -771,7 +771,9 @@ __device__ __forceinline__ void step_body(const RodDev& R, const Halo& H, float3
 }
 
 // Loads the rod's elements owned by thread tg of the rod (registers) and their joint
-// parameters (shared memory slot t, read back only by the same thread).
+// parameters (shared memory slot t, read back only by the same thread).  The last element's frame and
+// the last two joints do not exist: whatever the arrays hold there is not read (the branch-free
+// step multiplies it by zero, and nothing is stored there).
 template <int EPT, int NT>
 __device__ __forceinline__ void load_rod(const RodDev& R, const int t, const int tg, const float4* __restrict__ x4,
                                          const float4* __restrict__ v4, const float4* __restrict__ q4,
@@ -788,10 +790,10 @@ __device__ __forceinline__ void load_rod(const RodDev& R, const int t, const int
       r[e] = f3(a);
       w[e] = a.w;
       v[e] = f3(v4[R.off + i]);
-      q[e] = q4[R.off + i];
+      q[e] = i <= R.n - 2 ? q4[R.off + i] : make_float4(0.f, 0.f, 0.f, 1.f);
       om[e] = f3(o4[R.off + i]);
       if (par_u != nullptr) {
-        par_u[e * NT + t] = u4[R.off + i];
+        par_u[e * NT + t] = i <= R.n - 3 ? u4[R.off + i] : make_float4(0.f, 0.f, 0.f, 0.f);
         par_k[e * NT + t] = i <= R.n - 3 ? k4[R.off + i] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     } else {
@@ -1039,7 +1041,7 @@ __device__ __forceinline__ void run_rod(const RodDev& R, const Halo& H, const in
     if (i < R.n) {
       x4[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
       v4[R.off + i] = make_float4(v[e].x, v[e].y, v[e].z, 0.f);
-      q4[R.off + i] = q[e];
+      if (i <= R.n - 2) q4[R.off + i] = q[e];
       o4[R.off + i] = make_float4(om[e].x, om[e].y, om[e].z, 0.f);
       if (pos_out != nullptr) pos_out[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
     }

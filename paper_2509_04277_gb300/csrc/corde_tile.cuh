@@ -72,9 +72,9 @@ struct TileRod {
         r[e] = f3(a);
         w[e] = a.w;
         v[e] = f3(v4[R.off + i]);
-        q[e] = q4[R.off + i];
+        if (i <= n - 2) q[e] = q4[R.off + i];  // (what the arrays hold beyond the last frame and joint is not read)
         om[e] = f3(o4[R.off + i]);
-        if (i <= n - 3) {  // (a joint that does not exist has K = 0 and so no torques)
+        if (i <= n - 3) {  // (an absent joint has K = 0 and so no torques)
           uh[e] = f3(u4[R.off + i]);
           kk[e] = f3(k4[R.off + i]);
         }
@@ -257,7 +257,7 @@ struct TileRod {
       if (i < n) {
         x4[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
         v4[R.off + i] = make_float4(v[e].x, v[e].y, v[e].z, 0.f);
-        q4[R.off + i] = q[e];
+        if (i <= n - 2) q4[R.off + i] = q[e];
         o4[R.off + i] = make_float4(om[e].x, om[e].y, om[e].z, 0.f);
         if (pos_out != nullptr) pos_out[R.off + i] = make_float4(r[e].x, r[e].y, r[e].z, w[e]);
       }

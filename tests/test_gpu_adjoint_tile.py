@@ -84,3 +84,28 @@ def test_where_the_tiles_end(corde):
     c, ic = _grads(corde, [rod], 6, 3, True, budget=100000)  # one segment's records fit, all six steps' do not
     assert ic["mode"] == "recompute" or ic["blocks"] <= 2
     assert all(np.array_equal(a[k], c[k]) for k in a)
+
+
+def test_scratch_that_held_other_values(corde):
+    """Records and states live in scratch that is not cleared: a reverse pass after one that left
+    NaN there (a non-finite loss gradient and state) gives the gradients of a fresh handle."""
+    import torch
+
+    n_steps, every = 6, 3
+    rod = W.adjoint_rod(101, seed=8)
+    want, _ = _grads(corde, [rod], n_steps, every, True)
+    b = corde.RodBatch([rod])
+    drive = np.zeros((1, 8), np.float32)
+    drive[:, 0], drive[:, 6] = 0.02, 1.0
+    b.set_input(drive)
+    start = [torch.as_tensor(v, device="cuda") for v in b.state_numpy().values()]
+    corde.rod_set_state(b.handle, torch.full_like(start[0], float("nan")))
+    b.adjoint(torch.full_like(b.rollout(n_steps, every), float("nan")))
+    corde.rod_set_state(b.handle, *start)
+    traj = b.rollout(n_steps, every)
+    g = torch.zeros_like(traj)
+    g[:, :, :3] = 1e-2 * torch.cos(traj[:, :, :3] * 23.0)
+    got = {k: v.cpu().numpy() for k, v in b.adjoint(g).items()}
+    for k in got:
+        np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+    b.close()
