@@ -164,6 +164,8 @@ struct TileRoom {
 //    lane shorten the chain of a step (512 nodes: 2.15 against 2.88 us/step at four) and win up
 //    to seven warps a block over the largest cluster (2048 nodes: 2.73 against 2.98); longer rods
 //    take four (5000 nodes: 3.02 on a cluster, 3.62 at two on a grid).
+//    Beyond eight warps on every SM a grid's tiles take half the registers (131072 nodes: 7.0 us/step against 23.5 on
+//    the grid kernel).
 //  - Otherwise in one block of up to four tiles, while all rods' tiles find two warps per SM
 //    partition: 608 rods of 128 / 200 nodes 2.40 / 3.54 us/step against 3.46 / 4.03 as blocks, 304 of
 //    360 nodes 3.45 against 4.44; with more rods the repeated work loses (400 of 256: 5.64 / 3.90).
@@ -183,8 +185,9 @@ TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
     p.blocks = std::min(K, room->spare + 1);
   }
   p.warps = p.blocks > 0 ? (K + p.blocks - 1) / p.blocks : 0;
+  p.full = p.grid && p.warps > kTileMaxWarps;  // up to 16 warps on every SM
   const int64_t more = (int64_t)(p.blocks - 1) * count;
-  if (p.blocks >= 1 && p.warps <= kTileMaxWarps && !(p.grid && count > 1) && room->spare >= more) {
+  if (p.blocks >= 1 && p.warps <= (p.full ? 2 : 1) * kTileMaxWarps && !(p.grid && count > 1) && room->spare >= more) {
     room->spare -= (int)more;
     return p;
   }

@@ -147,6 +147,8 @@ TileFn tile_fn_t(const TilePlan& p) {
   return p.blocks > 1 ? tile_step_kernel<PER, ARITH, kTileCluster> : tile_step_kernel<PER, ARITH, kTileBlock>;
 }
 TileFn tile_fn(const TilePlan& p) {
+  if (p.full && p.grid && p.warps >= 1 && p.warps <= 2 * kTileMaxWarps && p.per == 4)
+    return p.arith == 4 ? tile_step_kernel<4, 4, kTileGrid, 512> : tile_step_kernel<4, 2, kTileGrid, 512>;
   if (p.warps < 1 || p.warps > kTileMaxWarps) return nullptr;
   if (p.full) {
     if (p.blocks != 1 || p.warps != 1) return nullptr;

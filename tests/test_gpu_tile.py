@@ -68,6 +68,23 @@ def test_long_rods(corde, n):
     _check(corde, [W.guidewire(n, seed=900 + n)], (1, 3))
 
 
+# more than eight warps on every SM (half the registers): the grid kernel, which several rods keep to
+def test_longest_rods(corde):
+    import torch
+
+    n = 100_001
+    rod = W.guidewire(n, seed=6)
+    a, b = corde.RodBatch([rod]), corde.RodBatch([rod, W.guidewire(n, seed=7)])
+    for steps in (1, 3):
+        a.step(steps)
+        b.step(steps)
+    sa, sb = a.state_numpy(), b.state_numpy()
+    assert all(np.array_equal(sa[k][:n].view(np.uint32), sb[k][:n].view(np.uint32)) for k in sa)
+    torch.cuda.synchronize()
+    a.close()
+    b.close()
+
+
 # iterations per exchange (10 and 11 fill the ghosts), velocity exchanges within a step beyond
 @pytest.mark.parametrize("iters", [0, 1, 2, 4, 5, 9, 10, 11, 12, 21, 22, 37])
 @pytest.mark.parametrize("n,plan", [(300, None), (300, (2, 256)), (4000, None)])
