@@ -485,7 +485,7 @@ def run_adjoint(args, torch, corde, W, n_rods=1):
             "launch": launch_info,
             "roofline_hbm": {"bytes": adj_bytes, "achieved_gbs": round(adj_bytes / (adj_ms * 1e-3) / 1e9, 2),
                              "peak_gbs": hbm, "frac": round(adj_bytes / (adj_ms * 1e-3) / 1e9 / hbm, 5),
-                             "note": "latency-bound like the forward: one block per rod"},
+                             "note": "latency-bound like the forward"},
             "fwd_ms": round(fwd_ms, 4), "fwd_launches": fwd_launches, "rollout_recorded_ms": round(roll_ms, 4),
             "adjoint_ms": round(adj_ms, 4), "adjoint_over_fwd": round(adj_ms / fwd_ms, 3),
             "adjoint_over_recorded_rollout": round(adj_ms / roll_ms, 3),
@@ -537,11 +537,10 @@ def run_pair(args, torch, corde, W, fp32):
     frac = {k: round(flops_step / (v * 1e-6) / 1e12 / peak, 7) for k, v in out.items()}
     sms = fp32["n_sms"]
     return {"unit": "us/step", "workload": "2 x 512 inextensible rods (catheter r=1 mm E=2 GPa, guidewire "
-                                           "r=0.45 mm E=60 GPa), one thread block per pair", "us_per_step": out,
+                                           "r=0.45 mm E=60 GPa), warp tiles that hold both rods", "us_per_step": out,
             "roofline_alu": {"flops_per_step": flops_step, "peak_tflops": round(peak, 2),
                              "peak_source": "measured (rod_fp32_peak, burst)",
-                             "frac_of_gpu": frac, "note": f"one pair = one thread block on one SM: at most 1/{sms} "
-                                                          f"of the GPU; x{sms} gives the fraction of that SM"},
+                             "frac_of_gpu": frac, "note": f"one pair on a few of {sms} SMs; latency-bound by design"},
             "cpu_oracle_us_per_step": cpu,
             "speedup_vs_oracle_1core_10ts": {f"v{m}": round(cpu[f"v{m}"] / out[f"v{m}_10ts"], 1) for m in (0, 1, 2)}}
 
@@ -874,13 +873,13 @@ def main_ours(args):
                          "unit": "TFLOP/s", "frac": round(achieved / fp32_peak, 8), "traffic": traffic,
                          "peak_source": "measured (rod_fp32_peak, burst: the kernel is timed alone)",
                          "fp32_peak": fp32,
-                         "note": f"one rod = one thread block on one of {n_sms} SMs; latency-bound by design",
-                         "kernel": "step_kernel<ept=%d, nt=%d>" % tuple(single["plan"]),
-                         "frac_of_one_sm": round(achieved / (fp32_peak / n_sms), 6),
+                         "note": f"one rod on a few of {n_sms} SMs (warp tiles, most lanes ghosts); latency-bound by "
+                                 "design",
+                         "kernel": "tile_step_kernel (plan ept=%d, nt=%d)" % tuple(single["plan"]),
                          "kernel_us_per_launch": round(single["kernel_ms_avg"] * 1e3, 3),
                          "duration": "timed region / launches (includes launch gaps); one launch bracketed "
                                      "alone by events: %.3f us" % (single["kernel_ms_isolated"] * 1e3)},
-            "latency": {"us_per_step": round(value, 4), "barriers_per_step": 2 + single["n_iters"],
+            "latency": {"us_per_step": round(value, 4), "barriers_per_step": 1,
                         "launch_overlap": "programmatic dependent launch (each launch waits in-kernel "
                                           "for the previous one's writes)",
                         "us_per_step_without_launch_overlap": round(single["us_per_step_without_launch_overlap"], 4),
@@ -888,8 +887,7 @@ def main_ours(args):
                         "haptic_1khz_realtime": bool(value * STEPS_PER_LAUNCH < 1000.0),
                         "floors_ns": {k: round(v, 2) for k, v in single["floors"].items()},
                         "step_over_grid_sync": round(value * 1e3 / single["floors"]["grid_sync_ns"], 3),
-                        "step_over_block_barrier_floor": round(
-                            value * 1e3 / ((2 + single["n_iters"]) * single["floors"]["block_ns"]), 3)},
+                        "step_over_cluster_barrier": round(value * 1e3 / single["floors"]["cluster8_ns"], 3)},
             "cpu_baseline": cpu,
             "clocks": single["clocks"],
             "checks": {"max_len_err": single["diag"][0], "max_qnorm_err": single["diag"][1],
@@ -966,7 +964,7 @@ def workload_config(world=1):
         "n_rods": 1, "n_elements": 512, "steps_per_launch": STEPS_PER_LAUNCH,
         "time_steps_per_bench_step": STEPS_PER_LAUNCH * LAUNCHES_PER_BENCH_STEP,
         "l2": "flushed (256 MiB write) between bench steps, outside the timed intervals",
-        "parallelism": f"replicas x{world}" if world > 1 else "single GPU, one thread block per rod",
+        "parallelism": f"replicas x{world}" if world > 1 else "single GPU, one rod over a cluster of warp tiles",
     }
 
 

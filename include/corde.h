@@ -214,7 +214,12 @@ int rod_diagnostics(rod_handle h, double* out);
  * hold; rod_autotune times the block variants that hold each length bin on the current
  * state (saved and restored) and keeps the fastest per bin.  rod_get_plan writes
  * [n_rods][3] ints (ept, nt, blocks; 0 = one block, C >= 2 a cluster of C blocks, -C a
- * cooperative grid of C blocks, see rod_set_plan_grid).  Synchronous. */
+ * cooperative grid of C blocks, see rod_set_plan_grid).  Synchronous.
+ * A plan fixes the arithmetic: the order in which an element's contributions are added and
+ * the form of the impulses follow from ept.  Without a mailbox, rods that leave SMs idle run
+ * as overlapping warp tiles over several of them, and rods of one tile as one warp, with the
+ * results of the plan bit for bit; rod_get_plan still reports the plan.  Tiles of a long rod
+ * meet at cluster or grid barriers of blocks that are resident together. */
 int rod_set_plan(rod_handle h, int ept, int nt);
 
 /* Launch overlap (on by default): the stepping kernels are launched with programmatic
@@ -366,9 +371,9 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
  * two, the copy of a step's records overlapping the reverse of the step after it),
  * threads per block, resident blocks per SM (occupancy API, with the launch's registers
  * and shared memory; 1 when pipelined), blocks of the launch (one per rod, two when
- * pipelined), the device's SMs, 1 when the records use the compact layout (see
- * rod_set_adjoint_record_budget), and 1 when the reverse pass was pipelined (see
- * rod_set_adjoint_pipeline); blocks / (blocks per SM x SMs), rounded up, is the number
+ * pipelined, one per four tiles of a rod on tiles), the device's SMs, 1 when the records use
+ * the compact layout (see rod_set_adjoint_record_budget), and 1 when the reverse pass of a rod
+ * ran over several blocks, pipelined or on tiles (see rod_set_adjoint_pipeline); blocks / (blocks per SM x SMs), rounded up, is the number
  * of waves.  Host-side only (zeros before the first rod_adjoint). */
 int rod_adjoint_info(rod_handle h, int* out);
 
@@ -391,7 +396,12 @@ int rod_adjoint_info(rod_handle h, int* out);
  * Host-side only. */
 int rod_set_adjoint_record_budget(rod_handle h, long long bytes);
 
-/* Pipelined reverse pass (enable != 0, the default).  A record-mode launch with the full
+/* Reverse pass of few rods (enable != 0, the default).
+ * Tiles: with at most 10 constraint iterations, every step's records and states within the
+ * record budget (per step and node 2 n_iters x 12 B and 64 B) and a block per four tiles of
+ * every rod finding an SM of its own (a rod of n nodes has about n / 20 tiles), all checkpoint
+ * segments are recorded at once and reversed on overlapping warp tiles.
+ * Pipelined, otherwise: a record-mode launch with the full
  * layout and two sweep buffers whose rods each find two free SMs (2 x rods <= SMs) runs
  * every rod on a cluster of two blocks: the first block records the checkpoint segments
  * (last first), the second reverses each one a segment later, so that recording and

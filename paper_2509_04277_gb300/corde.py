@@ -252,7 +252,7 @@ def rod_set_adjoint_record_budget(h, n_bytes):
 
 
 def rod_set_adjoint_pipeline(h, enable=True):
-    """Pipelined reverse pass (a cluster of two blocks per rod) where it applies."""
+    """Reverse pass over several blocks per rod (tiles, or a cluster of two blocks) where it applies."""
     _check(load().rod_set_adjoint_pipeline(h, 1 if enable else 0), "rod_set_adjoint_pipeline")
 
 

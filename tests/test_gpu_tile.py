@@ -125,3 +125,9 @@ def test_free_base(corde):
     rod.clamp = 0
     rod.gravity = (0.0, 0.0, -9.81)
     _check(corde, [rod], (1, 10))
+
+
+# a rod of tiles on a cooperative grid beside bins of other rods: the step is a graph of parallel branches
+@pytest.mark.parametrize("ns", [(20000, 300), (20000, 300, 300, 700), (11000, 20000, 5000)])
+def test_grid_of_tiles_beside_other_rods(corde, ns):
+    _check(corde, [W.guidewire(n, seed=n) for n in ns], (1, 10, 10))
