@@ -160,18 +160,18 @@ struct TileRoom {
 // elements per thread; per = 0 where the block, cluster or grid kernel runs.  Measured at 10 iterations:
 //  - Over several SMs while there are spare ones: the tiles repeat their ghosts' work (three times
 //    an element's at two elements per lane, 1.6 times at four).  One warp per SM partition is
-//    fastest (512 nodes: 2.15 us/step at 4 warps a block, 2.50 at 6, 2.59 at 8).  Two elements per
-//    lane shorten the chain of a step (512 nodes: 2.15 against 2.88 us/step at four) and win up
-//    to seven warps a block over the largest cluster (2048 nodes: 2.73 against 2.98); longer rods
-//    take four (5000 nodes: 3.02 on a cluster, 3.62 at two on a grid).
-//    Beyond eight warps on every SM a grid's tiles take half the registers (131072 nodes: 7.0 us/step against 23.5 on
-//    the grid kernel).
+//    fastest (512 nodes: 1.86 us/step at 4 warps a block, 2.24 at 6, 2.32 at 8; 2.29 as one block of
+//    the step kernel).  Two elements per lane shorten the chain of a step (512 nodes: 1.86 against
+//    2.33 us/step at four) and win up to seven warps a block over the largest cluster (2048 nodes:
+//    2.44 against 2.59, 6.20 as one block); longer rods take four (5000 nodes: 2.64 us/step, 6.57 on the
+//    cluster kernel).  Beyond eight warps on every SM a grid's tiles take half the registers (131072
+//    nodes: 7.0 us/step against 23.2 on the grid kernel).
 //  - Otherwise in one block of up to four tiles, while all rods' tiles find two warps per SM
-//    partition: 608 rods of 128 / 200 nodes 2.40 / 3.54 us/step against 3.46 / 4.03 as blocks, 304 of
-//    360 nodes 3.45 against 4.44; with more rods the repeated work loses (400 of 256: 5.64 / 3.90).
-//  - A rod of one tile repeats nothing: shuffles beat shared memory at any load, with the
-//    registers of 16 warps per SM (4864 rods of 64 nodes 5.53 us/step against 6.98, of 128 nodes
-//    11.1 against 11.4).
+//    partition: 304 rods of 128 / 200 / 360 nodes 1.98 / 2.17 / 3.23 us/step against 2.40 / 2.55 /
+//    3.65 as blocks, at most 3 % behind (608 of 200); with more rods the repeated work loses (400 of 256: 5.74 / 3.12), and
+//    with more than eight warps per SM so do single tiles of four elements per lane (4864 of 128: 11.1 / 10.0).
+//  - A rod of one tile of two elements per lane repeats nothing: shuffles beat shared memory at any
+//    load, with the registers of 16 warps per SM (4864 rods of 64 nodes 5.08 us/step against 5.42).
 TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   TilePlan p;
   p.arith = arith;
@@ -195,8 +195,8 @@ TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   p.blocks = 1;
   p.per = K2 == 1 ? 2 : 4;
   p.warps = K2 == 1 ? 1 : K4;
-  p.full = K2 == 1 || (K4 == 1 && room->saturated);
-  if (p.full ? (K2 > 1 && arith != 4) : (room->saturated || K4 > 4 || count > 8 / K4 * room->sms)) p.per = 0;
+  p.full = K2 == 1;
+  if (!p.full && (room->saturated || K4 > 4 || count > 8 / K4 * room->sms)) p.per = 0;
   return p;
 }
 

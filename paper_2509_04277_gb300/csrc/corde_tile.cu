@@ -151,9 +151,8 @@ TileFn tile_fn(const TilePlan& p) {
     return p.arith == 4 ? tile_step_kernel<4, 4, kTileGrid, 512> : tile_step_kernel<4, 2, kTileGrid, 512>;
   if (p.warps < 1 || p.warps > kTileMaxWarps) return nullptr;
   if (p.full) {
-    if (p.blocks != 1 || p.warps != 1) return nullptr;
-    if (p.per == 2) return p.arith == 4 ? tile_step_kernel<2, 4, kTileBlock, 512> : tile_step_kernel<2, 2, kTileBlock, 512>;
-    return p.arith == 4 ? tile_step_kernel<4, 4, kTileBlock, 512> : nullptr;
+    if (p.blocks != 1 || p.warps != 1 || p.per != 2) return nullptr;
+    return p.arith == 4 ? tile_step_kernel<2, 4, kTileBlock, 512> : tile_step_kernel<2, 2, kTileBlock, 512>;
   }
   if (p.per == 4 && p.arith == 4) return tile_fn_t<4, 4>(p);
   if (p.per == 4 && p.arith == 2) return tile_fn_t<4, 2>(p);

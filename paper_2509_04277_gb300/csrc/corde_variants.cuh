@@ -177,8 +177,8 @@ struct TilePlan {
   int per = 0;    // elements per lane (0: not a tile launch)
   int arith = 0;  // elements per thread of the layout whose arithmetic it repeats
   int blocks = 0, warps = 0;
-  bool full = false;  // the registers of 16 warps per SM: one-warp rods (two elements per lane, or four
-                      // with arith 4), or a grid of up to 16 warps per block (four per lane)
+  bool full = false;  // the registers of 16 warps per SM: one-warp rods (two elements per lane), or a grid of
+                      // up to 16 warps per block (four per lane)
   int grid = 0;   // the blocks form a cooperative grid (one rod; a.grid_halo: its exchange buffers), not a cluster
 };
 constexpr int kTileMaxWarps = 8;           // warps per block
