@@ -165,7 +165,7 @@ struct TileRoom {
 //    2.33 us/step at four) and win up to seven warps a block over the largest cluster (2048 nodes:
 //    2.44 against 2.59, 6.20 as one block); longer rods take four (5000 nodes: 2.64 us/step, 6.57 on the
 //    cluster kernel).  Beyond eight warps on every SM a grid's tiles take half the registers (131072
-//    nodes: 7.0 us/step against 23.2 on the grid kernel).
+//    nodes: 7.0 us/step against 23.2 on the grid kernel; 65536 4.5 against 24).
 //  - Otherwise in one block of up to four tiles, while all rods' tiles find two warps per SM
 //    partition: 304 rods of 128 / 200 / 360 nodes 1.98 / 2.17 / 3.23 us/step against 2.40 / 2.55 /
 //    3.65 as blocks, at most 3 % behind (608 of 200); with more rods the repeated work loses (400 of 256: 5.74 / 3.12), and
@@ -557,7 +557,11 @@ int build_bins(rod_handle h) {
       const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
       b.tile = tile_plan(nmax, b.count, arith, &room);
       if (b.tile.per) CK(prepare_tile(b.tile));
-      if (b.tile.per && b.tile.grid) CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
+      if (b.tile.per && b.tile.grid) {
+        CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
+        CK(cudaMemset(b.d_tile_gh, 0, tile_halo_bytes(b.tile.per, nmax)));  // no stamps
+        CK(cudaStreamSynchronize(cudaStreamLegacy));  // before a launch on a stream that doesn't wait for this one
+      }
     }
     h->bins.push_back(b);
   }

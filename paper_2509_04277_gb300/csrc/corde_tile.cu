@@ -7,7 +7,7 @@
 // neighbour: the force phase spoils one element from the tile's edge inward, each constraint
 // iteration two more, 2 n_iters + 1 a step.  G lanes hold 24 (PER 4) or 22 (PER 2)
 // elements, so the paper's ten iterations fit, and one exchange of the ghosts' state per
-// step, with one barrier, replaces the twelve.  Fewer iterations allow several steps per
+// step, with one barrier (on a grid: a wait for the two neighbours), replaces the twelve.  Fewer iterations allow several steps per
 // exchange; more need velocity exchanges within the step.
 //
 // Every element takes the arithmetic of the <ARITH, *> layout of the block kernels, in
@@ -35,12 +35,12 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
   const RodDev R = rods[rid];
   // the work list and the rod constants are only written with the host waiting, so they are
   // read before the wait for the stream's previous kernel (0.03 us a step of ten-step launches)
-  if constexpr (SYNC != kTileGrid) pdl_begin();
+  if constexpr (!tile_on_grid(SYNC)) pdl_begin();
   const int K = T::count(R.n);
   const int k = (blockIdx.x % C) * W + (threadIdx.x >> 5);  // this warp's tile
   const bool active = k < K;  // warps beyond the rod only take part in the barriers
   TileRod<PER, ARITH> rod(R, lane, active ? (k * T::O + lane) * PER : R.n, x4, v4, q4, o4, u4, k4);
-  TileLink<PER, SYNC, T::kBuf> link(k, K, W, lane, (R.n + PER - 1) / PER, smem, gh);
+  TileLink<PER, SYNC, SYNC == kTileGrid ? T::kGridBuf : T::kBuf> link(k, K, W, lane, (R.n + PER - 1) / PER, smem, gh);
   float3 v_drive = zero3(), w_drive = zero3();
   if (drive != nullptr) {
     v_drive = f3(drive[2 * rid]);
@@ -135,6 +135,8 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
   // every tile has loaded its ghosts' elements, and read its neighbours' last buffers, before
   // any state is overwritten or any block leaves
   if (K > 1) link.barrier();
+  link.leave(k, lane, gh);
+  if (link.lost) rod.spoil();
   if (link.owned) rod.store(x4, v4, q4, o4, pos_out);
 }
 
@@ -143,12 +145,13 @@ using TileFn = void (*)(const RodDev*, const int*, float4*, float4*, float4*, fl
 
 template <int PER, int ARITH>
 TileFn tile_fn_t(const TilePlan& p) {
-  if (p.grid) return tile_step_kernel<PER, ARITH, kTileGrid>;
+  if constexpr (PER == 4)
+    if (p.grid) return tile_step_kernel<PER, ARITH, kTileGrid>;
   return p.blocks > 1 ? tile_step_kernel<PER, ARITH, kTileCluster> : tile_step_kernel<PER, ARITH, kTileBlock>;
 }
 TileFn tile_fn(const TilePlan& p) {
   if (p.full && p.grid && p.warps >= 1 && p.warps <= 2 * kTileMaxWarps && p.per == 4)
-    return p.arith == 4 ? tile_step_kernel<4, 4, kTileGrid, 512> : tile_step_kernel<4, 2, kTileGrid, 512>;
+    return p.arith == 4 ? tile_step_kernel<4, 4, kTileGridSync, 512> : tile_step_kernel<4, 2, kTileGridSync, 512>;
   if (p.warps < 1 || p.warps > kTileMaxWarps) return nullptr;
   if (p.full) {
     if (p.blocks != 1 || p.warps != 1 || p.per != 2) return nullptr;
@@ -169,7 +172,8 @@ int tile_smem(const TilePlan& p, int warps) {
 
 int tile_count(int per, int n) { return per == 4 ? Tile<4>::count(n) : Tile<2>::count(n); }
 int64_t tile_halo_bytes(int per, int n) {
-  return (int64_t)2 * tile_count(per, n) * (per == 4 ? Tile<4>::kBuf : Tile<2>::kBuf) * (int64_t)sizeof(float4);
+  const int64_t buf = per == 4 ? Tile<4>::kGridBuf : Tile<2>::kGridBuf;
+  return (2 * tile_count(per, n) * buf + 1) * (int64_t)sizeof(float4);  // and the last stamp
 }
 
 cudaError_t prepare_tile(const TilePlan& p) {

@@ -18,6 +18,7 @@ struct Tile {
   static constexpr int SLOTS = PER == 4 ? 13 : 7;    // float4 of a lane's state: 13 floats per element
   static constexpr int VSLOTS = (3 * PER + 3) / 4;   // float4 of its velocities
   static constexpr int kBuf = SLOTS * 32;            // float4 of a tile's exchange buffer
+  static constexpr int kGridBuf = (4 * SLOTS + 2) / 3 * 32;  // the same on a grid: three floats and a stamp
   // tiles of Q lanes' worth of elements
   __host__ __device__ static int count_lanes(int Q) { return Q <= 32 ? 1 : (Q - 32 + O - 1) / O + 1; }
   // tiles of a rod of n nodes
@@ -249,6 +250,15 @@ struct TileRod {
     for (int e = 0; e < PER; ++e) v[e] = f3(f[3 * e], f[3 * e + 1], f[3 * e + 2]);
   }
 
+  // a state that no one takes for a result
+  __device__ __forceinline__ void spoil() {
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      const float nan = __int_as_float(0x7fffffff);
+      r[e] = v[e] = f3(nan, nan, nan);
+    }
+  }
+
   __device__ __forceinline__ void store(float4* __restrict__ x4, float4* __restrict__ v4, float4* __restrict__ q4,
                                         float4* __restrict__ o4, float4* __restrict__ pos_out) const {
 #pragma unroll
@@ -267,7 +277,36 @@ struct TileRod {
 
 // How a rod's tiles exchange: the block's shared memory and barrier; the shared memory of a
 // cluster's blocks and its barrier; global memory and a grid sync.
-enum TileSync { kTileBlock, kTileCluster, kTileGrid };
+// kTileGrid: neighbours wait for each other by polling the data (a step of 16384 / 65536 nodes 3.31 /
+// 4.51 us, 3.92 / 5.02 with a grid barrier between writing and reading; polling one slot and then reading all
+// 3.65 / 4.53).  kTileGridSync: the barrier, with more than eight warps per SM, where the loop's
+// registers spill (131072 nodes 7.01 us against 7.63).
+enum TileSync { kTileBlock, kTileCluster, kTileGrid, kTileGridSync };
+__host__ __device__ constexpr bool tile_on_grid(int sync) { return sync == kTileGrid || sync == kTileGridSync; }
+
+// 16 bytes of three floats and a stamp in L2, written and read as one: a reader that finds the
+// stamp has the floats, so neighbours need no barrier and no fence between data and flag.
+__device__ __forceinline__ void put_stamped(float4* p, float x, float y, float z, unsigned stamp) {
+  asm volatile(
+      "{ .reg .b128 t; .reg .b64 lo, hi; mov.b64 lo, {%1, %2}; mov.b64 hi, {%3, %4}; mov.b128 t, {lo, hi};\n\t"
+      "st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p), "r"(__float_as_uint(x)), "r"(__float_as_uint(y)),
+      "r"(__float_as_uint(z)), "r"(stamp)
+      : "memory");
+}
+__device__ __forceinline__ unsigned get_stamped(const float4* p, float& x, float& y, float& z) {
+  unsigned a, b, c, stamp;
+  asm volatile(
+      "{ .reg .b128 t; .reg .b64 lo, hi; ld.relaxed.gpu.global.b128 t, [%4];\n\t"
+      "mov.b128 {lo, hi}, t; mov.b64 {%0, %1}, lo; mov.b64 {%2, %3}, hi; }"
+      : "=r"(a), "=r"(b), "=r"(c), "=r"(stamp)
+      : "l"(p)
+      : "memory");
+  x = __uint_as_float(a);
+  y = __uint_as_float(b);
+  z = __uint_as_float(c);
+  return stamp;
+}
+constexpr int kTileSpinLimit = 1 << 22;  // polls before a wait for a neighbour gives up (seconds)
 
 // A warp's place among the K tiles of a rod (or pair): tile k holds lanes k O ... k O + 31 of it.
 // BUF: float4 of a tile's exchange buffer, of which there are two, used in turn.
@@ -278,6 +317,10 @@ struct TileLink {
   const float4* theirs;     // where a ghost lane's owner publishes (NULL: not a ghost)
   int64_t stride;           // from one buffer to the other
   int parity = 0;
+  // grids: the stamp of the last exchange (it goes on from launch to launch, kept behind the buffers), and
+  // whether a wait has given up
+  unsigned stamp = 0;
+  bool lost = false;
 
   // Q: lanes of the whole rod; smem: the block's buffers, or gh: the grid's
   __device__ __forceinline__ TileLink(int k, int K, int W, int lane, int Q, float4* smem, float4* gh) {
@@ -285,13 +328,14 @@ struct TileLink {
     const bool active = k < K;
     const int g = k * T::O + lane, wid = threadIdx.x >> 5;
     owned = active && (k == 0 || lane >= T::G) && (k == K - 1 || lane < 32 - T::G);
-    mine = SYNC == kTileGrid ? gh + (int64_t)k * BUF + lane : smem + wid * BUF + lane;
-    stride = (int64_t)(SYNC == kTileGrid ? K : W) * BUF;
+    mine = tile_on_grid(SYNC) ? gh + (int64_t)k * BUF + lane : smem + wid * BUF + lane;
+    stride = (int64_t)(tile_on_grid(SYNC) ? K : W) * BUF;
     theirs = nullptr;
+    if constexpr (SYNC == kTileGrid) stamp = __ldcg(reinterpret_cast<const unsigned*>(gh + 2 * stride));
     if (active && !owned && g < Q) {
       const int ok = min(max((g - T::G) / T::O, 0), K - 1);  // the tile that owns lane g
       const int ol = g - ok * T::O;
-      if constexpr (SYNC == kTileGrid) {
+      if constexpr (tile_on_grid(SYNC)) {
         theirs = gh + (int64_t)ok * BUF + ol;
       } else if constexpr (SYNC == kTileCluster) {
         theirs = cooperative_groups::this_cluster().map_shared_rank(smem + (ok % W) * BUF + ol, ok / W);
@@ -301,7 +345,7 @@ struct TileLink {
     }
   }
   __device__ __forceinline__ void barrier() const {
-    if constexpr (SYNC == kTileGrid) {
+    if constexpr (tile_on_grid(SYNC)) {
       cooperative_groups::this_grid().sync();
     } else if constexpr (SYNC == kTileCluster) {
       cooperative_groups::this_cluster().sync();
@@ -309,7 +353,7 @@ struct TileLink {
       __syncthreads();
     }
   }
-  // the barrier of an exchange: it orders the tiles' shared-memory buffers (global memory on a grid)
+  // the barrier of an exchange: it orders the tiles' shared-memory buffers (global memory on a grid of many warps)
   // and nothing else.  The full cluster barrier also waits for a block's global accesses in
   // flight, the adjoint's prefetches above all.
   __device__ __forceinline__ void meet() const {
@@ -324,12 +368,13 @@ struct TileLink {
   // ghost lanes receive the N float4 of the lane that owns their elements (true for them)
   template <int N>
   __device__ __forceinline__ bool trade(float4 (&a)[N]) {
-    static_assert(N * 32 <= BUF, "exchange buffer");
+    if constexpr (SYNC == kTileGrid) return trade_stamped(a);
+    static_assert(SYNC == kTileGrid || N * 32 <= BUF, "exchange buffer");
     if (owned) {
       float4* m = mine + parity * stride;
 #pragma unroll
       for (int s = 0; s < N; ++s) {
-        if constexpr (SYNC == kTileGrid) __stcg(m + s * 32, a[s]);
+        if constexpr (SYNC == kTileGridSync) __stcg(m + s * 32, a[s]);
         else m[s * 32] = a[s];
       }
     }
@@ -338,12 +383,55 @@ struct TileLink {
       const float4* p = theirs + parity * stride;
 #pragma unroll
       for (int s = 0; s < N; ++s) {
-        if constexpr (SYNC == kTileGrid) a[s] = __ldcg(p + s * 32);
+        if constexpr (SYNC == kTileGridSync) a[s] = __ldcg(p + s * 32);
         else a[s] = p[s * 32];
       }
     }
     parity ^= 1;
     return theirs != nullptr;
+  }
+  // On a grid a tile waits for its two neighbours only, by polling the data itself.  A tile
+  // publishes exchange i only after it has read its neighbours' exchange i - 1, and they published
+  // that after they had read its exchange i - 2: two buffers suffice.
+  template <int N>
+  __device__ __forceinline__ bool trade_stamped(float4 (&a)[N]) {
+    constexpr int M = (4 * N + 2) / 3;
+    float f[3 * M];
+    f[3 * M - 1] = f[3 * M - 2] = 0.f;
+#pragma unroll
+    for (int s = 0; s < N; ++s) {
+      f[4 * s] = a[s].x;
+      f[4 * s + 1] = a[s].y;
+      f[4 * s + 2] = a[s].z;
+      f[4 * s + 3] = a[s].w;
+    }
+    ++stamp;
+    if (owned) {
+      float4* m = mine + parity * stride;
+#pragma unroll
+      for (int s = 0; s < M; ++s) put_stamped(m + s * 32, f[3 * s], f[3 * s + 1], f[3 * s + 2], stamp);
+    }
+    const float4* p = theirs + parity * stride;
+    for (int tries = 0;; ++tries) {
+      unsigned other = 0;
+      if (theirs != nullptr) {
+#pragma unroll
+        for (int s = 0; s < M; ++s) other |= get_stamped(p + s * 32, f[3 * s], f[3 * s + 1], f[3 * s + 2]) ^ stamp;
+      }
+      if (__all_sync(0xffffffffu, other == 0)) break;
+      if (lost || tries == kTileSpinLimit) {
+        lost = true;
+        break;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < N; ++s) a[s] = make_float4(f[4 * s], f[4 * s + 1], f[4 * s + 2], f[4 * s + 3]);
+    parity ^= 1;
+    return theirs != nullptr;
+  }
+  // after the launch's last barrier: the stamps go on from here
+  __device__ __forceinline__ void leave(int k, int lane, float4* gh) const {
+    if (SYNC == kTileGrid && k == 0 && lane == 0) *reinterpret_cast<unsigned*>(gh + 2 * stride) = stamp;
   }
 };
 

@@ -131,3 +131,11 @@ def test_free_base(corde):
 @pytest.mark.parametrize("ns", [(20000, 300), (20000, 300, 300, 700), (11000, 20000, 5000)])
 def test_grid_of_tiles_beside_other_rods(corde, ns):
     _check(corde, [W.guidewire(n, seed=n) for n in ns], (1, 10, 10))
+
+
+# tiles on a grid wait for their neighbours' data: several exchanges a step, one in several steps, call after call
+@pytest.mark.parametrize("n,iters", [(12000, 0), (12000, 4), (12000, 25), (32768, 12)])
+def test_grid_exchanges(corde, n, iters):
+    rod = W.guidewire(n, seed=iters)
+    rod.n_iters = iters
+    _check(corde, [rod], (1, 12, 1, 7, 30))
