@@ -222,6 +222,24 @@ int rod_diagnostics(rod_handle h, double* out);
  * meet at cluster or grid barriers of blocks that are resident together. */
 int rod_set_plan(rod_handle h, int ept, int nt);
 
+/* Warp tiles (on by default): enable = 0 keeps every rod, pair and reverse pass on the block,
+ * cluster and grid kernels of its plan, with the same results bit for bit.  enable must be
+ * 0 or 1 (CORDE_ERR_ARG otherwise).  Synchronous. */
+int rod_set_tiles(rod_handle h, int enable);
+
+/* The kernel that steps each rod: out [n_rods][4] ints = one of the kinds below, blocks per rod
+ * (or pair), threads per block, elements per thread (per lane on tiles).  With a mailbox
+ * enabled, that of a mailbox launch.  Host-side only. */
+#define CORDE_KERNEL_BLOCK 0       /* one block */
+#define CORDE_KERNEL_CLUSTER 1     /* a cluster of blocks */
+#define CORDE_KERNEL_GRID 2        /* a cooperative grid of blocks */
+#define CORDE_KERNEL_SELF 3        /* the self-collision block */
+#define CORDE_KERNEL_PAIR 4        /* both rods of a pair in one block */
+#define CORDE_KERNEL_TILES 5       /* warp tiles of one block or cluster */
+#define CORDE_KERNEL_TILES_GRID 6  /* warp tiles of a cooperative grid */
+#define CORDE_KERNEL_PAIR_TILES 7  /* warp tiles that hold both rods of a pair */
+int rod_get_kernels(rod_handle h, int* out);
+
 /* Launch overlap (on by default): the stepping kernels are launched with programmatic
  * stream serialisation, so a launch is scheduled while the stream's previous stepping
  * kernel still runs and starts stepping as soon as that kernel's writes are visible (each
@@ -376,6 +394,11 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
  * ran over several blocks, pipelined or on tiles (see rod_set_adjoint_pipeline); blocks / (blocks per SM x SMs), rounded up, is the number
  * of waves.  Host-side only (zeros before the first rod_adjoint). */
 int rod_adjoint_info(rod_handle h, int* out);
+
+/* Reverse launches of the last rod_adjoint by kernel: out [3] ints = one block per rod,
+ * pipelined over two blocks, warp tiles (recording and reverse count as one).  Host-side
+ * only (zeros before the first rod_adjoint). */
+int rod_adjoint_kernels(rod_handle h, int* out);
 
 /* Scratch budget of rod_adjoint's record mode (default 1 GiB).  Within a checkpoint
  * segment the reverse pass needs every step's velocities before each constraint

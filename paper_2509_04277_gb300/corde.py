@@ -61,6 +61,9 @@ SIGNATURES = {
     "rod_set_material": (ctypes.c_int, [_VP, _VP, _VP]),
     "rod_diagnostics": (ctypes.c_int, [_VP, _VP]),
     "rod_set_plan": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int]),
+    "rod_set_tiles": (ctypes.c_int, [_VP, ctypes.c_int]),
+    "rod_get_kernels": (ctypes.c_int, [_VP, _VP]),
+    "rod_adjoint_kernels": (ctypes.c_int, [_VP, _VP]),
     "rod_set_launch_overlap": (ctypes.c_int, [_VP, ctypes.c_int]),
     "rod_set_adjoint_record_budget": (ctypes.c_int, [_VP, ctypes.c_longlong]),
     "rod_set_adjoint_pipeline": (ctypes.c_int, [_VP, ctypes.c_int]),
@@ -254,6 +257,25 @@ def rod_set_adjoint_record_budget(h, n_bytes):
 def rod_set_adjoint_pipeline(h, enable=True):
     """Reverse pass over several blocks per rod (tiles, or a cluster of two blocks) where it applies."""
     _check(load().rod_set_adjoint_pipeline(h, 1 if enable else 0), "rod_set_adjoint_pipeline")
+
+
+def rod_set_tiles(h, enable=True):
+    """Warp tiles where they apply (default), or the block, cluster and grid kernels of the plans."""
+    _check(load().rod_set_tiles(h, int(enable)), "rod_set_tiles")
+
+
+KERNEL_KINDS = ("block", "cluster", "grid", "self", "pair", "tiles", "tiles_grid", "pair_tiles")
+
+
+def rod_get_kernels(h, out):
+    _check(load().rod_get_kernels(h, _ptr(out)), "rod_get_kernels")
+
+
+def rod_adjoint_kernels(h) -> dict:
+    """Reverse launches of the last rod_adjoint by kernel."""
+    out = np.zeros(3, dtype=np.int32)
+    _check(load().rod_adjoint_kernels(h, out.ctypes.data), "rod_adjoint_kernels")
+    return {"block": int(out[0]), "pipelined": int(out[1]), "tiles": int(out[2])}
 
 
 def rod_set_launch_overlap(h, enable):
@@ -550,6 +572,15 @@ class RodBatch:
         out = np.zeros((self.n_rods, 3), dtype=np.int32)
         rod_get_plan(self.handle, out)
         return out
+
+    def set_tiles(self, enable: bool):
+        rod_set_tiles(self.handle, 1 if enable else 0)
+
+    def kernels(self) -> list:
+        """Per rod: (kind, blocks, threads per block, elements per thread or lane) of the kernel that steps it."""
+        out = np.zeros((self.n_rods, 4), dtype=np.int32)
+        rod_get_kernels(self.handle, out)
+        return [(KERNEL_KINDS[k[0]], int(k[1]), int(k[2]), int(k[3])) for k in out]
 
     def set_plan_cluster(self, ept, nt, cluster):
         rod_set_plan_cluster(self.handle, ept, nt, cluster)

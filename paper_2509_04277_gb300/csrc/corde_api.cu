@@ -147,6 +147,7 @@ struct Bin {
   const StepVariant* trim = nullptr;  // the smaller block that holds the bin's rods
   TilePlan tile;           // per > 0: launches without a mailbox run the tile kernel
   float4* d_tile_gh = nullptr;  // tiles on a cooperative grid: their exchange buffers
+  std::vector<int> rods;        // the bin's rods, in the order of d_work
 };
 
 // How much of the GPU a handle's rods leave free (see tile_plan).
@@ -224,6 +225,7 @@ struct corde_rods {
   std::vector<Bin> bins;
   int last_launches = 0;
   int pdl = 1;  // stepping kernels launched with programmatic stream serialisation
+  int tiles = 1;  // warp tiles where they apply (rod_set_tiles)
   // rollout / adjoint
   float4* d_ckpt = nullptr;  // [n_ckpt][4][E]
   size_t ckpt_cap = 0;       // float4 entries
@@ -236,6 +238,7 @@ struct corde_rods {
   // last rod_adjoint's largest launch: mode, nt, blocks/SM, blocks, SMs, compact records,
   // pipelined
   int adj_info[7] = {0, 0, 0, 0, 0, 0, 0};
+  int adj_kernels[3] = {0, 0, 0};  // launches of the last rod_adjoint: block kernel, pipelined, tiles
   int adj_pipe = 1;  // pipelined reverse where it applies (rod_set_adjoint_pipeline)
   std::vector<Bin> adj_bins;  // variant = threads per block
   // catheter/guidewire pairs
@@ -547,12 +550,13 @@ int build_bins(rod_handle h) {
     for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
+    b.rods = rods;
     if (b.grid) {
       const size_t n4 = rods.size() * 2 * (size_t)b.cluster * kHaloSlots * 2;
       CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
       CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
     }
-    if (b.cluster >= 0) {
+    if (b.cluster >= 0 && h->tiles) {
       const int nmax = b.n_max;
       const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
       b.tile = tile_plan(nmax, b.count, arith, &room);
@@ -1315,7 +1319,7 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         if (v.capacity() >= 8 * nmax && v.nt > 32) continue;  // mostly idle threads
         std::vector<Bin> one{Bin{(int)vi, (int)rods.size(), d_work}};
         TileRoom room = tile_room(h);
-        one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
+        if (h->tiles) one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
         if (one[0].tile.per && prepare_tile(one[0].tile) != cudaSuccess) one[0].tile.per = 0;
         restore();
         if ((rc = launch_bins(h, one, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
@@ -1452,6 +1456,11 @@ int rod_self_collision_stats(rod_handle h, int rod, int* out) {
   return CORDE_OK;
 }
 
+static void free_adjoint_bins(rod_handle h) {
+  for (auto& b : h->adj_bins) cudaFree(b.d_work);
+  h->adj_bins.clear();
+}
+
 // Pair kernel layout: two elements per thread up to 512 nodes per rod, four up to 1024,
 // the smallest power-of-two group (>= 32 threads) holding the longer rod.
 static int pair_layout(int n, int* ept, int* nt) {
@@ -1484,7 +1493,7 @@ static int build_pair_bins(rod_handle h) {
       pb.tile.arith = ept;
       pb.tile.blocks = std::min((K + 3) / 4, kMaxCluster);
       pb.tile.warps = (K + pb.tile.blocks - 1) / pb.tile.blocks;
-      if (pb.tile.warps <= kTileMaxWarps && (int64_t)pb.tile.blocks * pb.count + h->n_rods <= h->sms) {
+      if (h->tiles && pb.tile.warps <= kTileMaxWarps && (int64_t)pb.tile.blocks * pb.count + h->n_rods <= h->sms) {
         CK(prepare_pair_tile(pb.tile, pb.two_way));
         pb.tile.per = 2;
       }
@@ -1520,6 +1529,50 @@ int rod_bind(rod_handle h, int outer, int inner, int mode) {
   return build_pair_bins(h);
 }
 
+int rod_set_tiles(rod_handle h, int enable) {
+  if (int rc = check_handle(h)) return rc;
+  if (enable != 0 && enable != 1) return fail(CORDE_ERR_ARG, "rod_set_tiles: enable must be 0 or 1");
+  if (h->tiles == enable) return CORDE_OK;
+  h->tiles = enable;
+  free_adjoint_bins(h);  // (built again by the next rod_rollout or rod_adjoint)
+  if (int rc = build_bins(h)) return rc;
+  return h->pairs.empty() ? CORDE_OK : build_pair_bins(h);
+}
+
+int rod_get_kernels(rod_handle h, int* out) {
+  if (!h || !out) return fail(CORDE_ERR_ARG, "rod_get_kernels: NULL argument");
+  auto put = [&](int r, int kind, int blocks, int threads, int per) {
+    const int k[4] = {kind, blocks, threads, per};
+    std::copy(k, k + 4, out + 4 * r);
+  };
+  const bool tiles = h->mb_period == 0;
+  for (const Bin& b : h->bins)
+    for (int r : b.rods) {
+      if (b.tile.per && tiles) {
+        put(r, b.tile.grid ? CORDE_KERNEL_TILES_GRID : CORDE_KERNEL_TILES, b.tile.blocks, 32 * b.tile.warps, b.tile.per);
+      } else if (b.cluster < 0) {
+        put(r, CORDE_KERNEL_SELF, 1, kSelfVariants[b.variant].nt, kSelfVariants[b.variant].ept);
+      } else if (b.cluster > 0) {
+        const ClusterVariant& v = kClusterVariants[b.variant];
+        put(r, b.grid ? CORDE_KERNEL_GRID : CORDE_KERNEL_CLUSTER, b.cluster, v.nt, v.ept);
+      } else {
+        const StepVariant& v = b.trim ? *b.trim : variants()[b.variant];
+        put(r, CORDE_KERNEL_BLOCK, 1, v.nt, v.ept);
+      }
+    }
+  for (const int4& p : h->pairs) {
+    int ept = 0, nt = 0;
+    pair_layout(std::max(h->n_nodes[p.x], h->n_nodes[p.y]), &ept, &nt);
+    for (const auto& pb : h->pair_bins)
+      if (pb.ept == ept && pb.nt == nt)
+        for (int r : {p.x, p.y}) {
+          if (pb.tile.per && tiles) put(r, CORDE_KERNEL_PAIR_TILES, pb.tile.blocks, 32 * pb.tile.warps, pb.tile.per);
+          else put(r, CORDE_KERNEL_PAIR, 1, 2 * nt, ept);
+        }
+  }
+  return CORDE_OK;
+}
+
 // Bins of the adjoint layout: two elements per thread, the smallest power-of-two block
 // (>= 32 threads) holding the rod.  Bin.variant is the index of the matching <2, nt> step
 // variant, so that rod_rollout and the adjoint's recomputation run the same kernel code.
@@ -1540,7 +1593,7 @@ static int build_adjoint_bins(rod_handle h) {
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
     CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
     for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
-    b.tile = tile_plan(b.n_max, b.count, 2, &room);
+    if (h->tiles) b.tile = tile_plan(b.n_max, b.count, 2, &room);
     // two or more tiles in one block don't pay here: a training step of 256 rods of 256 nodes took
     // 2.77 ms against 2.65 with the block kernel, though the rollout alone is no slower
     if (b.tile.blocks == 1 && b.tile.warps > 1 && b.count > h->sms) b.tile.per = 0;
@@ -1652,7 +1705,7 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   std::vector<int> tile_blocks(h->adj_bins.size(), 0);
   size_t sweep_need = 0, seg_need = 0;
   int spare = sms - h->n_rods;
-  for (size_t i = 0; i < h->adj_bins.size() && h->adj_pipe && iters <= kAdjointTileIters; ++i) {
+  for (size_t i = 0; i < h->adj_bins.size() && h->tiles && h->adj_pipe && iters <= kAdjointTileIters; ++i) {
     const Bin& b = h->adj_bins[i];
     const int blocks = (tile_count(2, b.n_max) + 3) / 4;
     const size_t rec = (size_t)h->ro_steps * b.count * 2 * iters * 3 * adjoint_tile_npad(b.n_max) / 4;  // float4
@@ -1730,6 +1783,7 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   a.domega0 = dev_out[5];
   int launches = 0;
   std::fill(h->adj_info, h->adj_info + 7, 0);
+  std::fill(h->adj_kernels, h->adj_kernels + 3, 0);
   for (size_t i = 0; i < h->adj_bins.size(); ++i) {
     const Bin& b = h->adj_bins[i];
     const int nt = variants()[b.variant].nt;
@@ -1765,6 +1819,7 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
       cudaError_t e = launch_adjoint_tile(t, warps, s);
       if (e != cudaSuccess) return fail(CORDE_ERR_CUDA, std::string("adjoint tile launch: ") + cudaGetErrorString(e));
       launches += 2;
+      ++h->adj_kernels[2];
       continue;
     }
     int smem = adjoint_smem_bytes(nt, iters, mode[i], compact[i] != 0);
@@ -1789,6 +1844,7 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
                             : launch_adjoint(nt, mode[i], compact[i] != 0, a, b.count, smem, s);
     if (e != cudaSuccess) return fail(CORDE_ERR_CUDA, std::string("adjoint launch: ") + cudaGetErrorString(e));
     ++launches;
+    ++h->adj_kernels[pipe[i] ? 1 : 0];
   }
   h->last_launches = launches;
   return CORDE_OK;
@@ -1797,6 +1853,12 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
 int rod_adjoint_info(rod_handle h, int* out) {
   if (!h || !out) return fail(CORDE_ERR_ARG, "rod_adjoint_info: NULL argument");
   std::copy(h->adj_info, h->adj_info + 7, out);
+  return CORDE_OK;
+}
+
+int rod_adjoint_kernels(rod_handle h, int* out) {
+  if (!h || !out) return fail(CORDE_ERR_ARG, "rod_adjoint_kernels: NULL argument");
+  std::copy(h->adj_kernels, h->adj_kernels + 3, out);
   return CORDE_OK;
 }
 
@@ -2049,7 +2111,7 @@ void rod_destroy(rod_handle h) {
   cudaFree(h->d_drive); cudaFree(h->d_elem_rod); cudaFree(h->d_drive_graph);
   cudaFree(h->d_ckpt); cudaFree(h->d_seg); cudaFree(h->d_self_stats); cudaFree(h->d_self_skin);
   cudaFree(h->d_sweep_rec);
-  for (auto& b : h->adj_bins) cudaFree(b.d_work);
+  free_adjoint_bins(h);
   for (auto& pb : h->pair_bins) cudaFree(pb.d_pairs);
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   for (auto st : h->side) cudaStreamDestroy(st);
