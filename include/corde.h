@@ -227,6 +227,15 @@ int rod_set_plan(rod_handle h, int ept, int nt);
  * 0 or 1 (CORDE_ERR_ARG otherwise).  Synchronous. */
 int rod_set_tiles(rod_handle h, int enable);
 
+/* Warp tiles on a cooperative grid (CORDE_KERNEL_TILES_GRID) wait for their neighbours' data, each
+ * wait for at most `polls` reads (default 2^22, seconds).  A wait that runs out ends the others of
+ * the launch too; the launch ends, and the whole rod's state, positions output and trajectory rows
+ * of that launch are NaN.  The step's call has then returned CORDE_OK (launches are asynchronous):
+ * rod_wait_status gives the number of rods to which this happened since the last rod_wait_status,
+ * and rod_diagnostics reports them as non-finite.  Both are synchronous. */
+int rod_set_wait_limit(rod_handle h, unsigned polls);
+int rod_wait_status(rod_handle h, int* n_lost);
+
 /* The kernel that steps each rod: out [n_rods][4] ints = one of the kinds below, blocks per rod
  * (or pair), threads per block, elements per thread (per lane on tiles).  With a mailbox
  * enabled, that of a mailbox launch.  Host-side only. */

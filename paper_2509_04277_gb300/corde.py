@@ -62,6 +62,8 @@ SIGNATURES = {
     "rod_diagnostics": (ctypes.c_int, [_VP, _VP]),
     "rod_set_plan": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int]),
     "rod_set_tiles": (ctypes.c_int, [_VP, ctypes.c_int]),
+    "rod_set_wait_limit": (ctypes.c_int, [_VP, ctypes.c_uint]),
+    "rod_wait_status": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_int)]),
     "rod_get_kernels": (ctypes.c_int, [_VP, _VP]),
     "rod_adjoint_kernels": (ctypes.c_int, [_VP, _VP]),
     "rod_set_launch_overlap": (ctypes.c_int, [_VP, ctypes.c_int]),
@@ -262,6 +264,17 @@ def rod_set_adjoint_pipeline(h, enable=True):
 def rod_set_tiles(h, enable=True):
     """Warp tiles where they apply (default), or the block, cluster and grid kernels of the plans."""
     _check(load().rod_set_tiles(h, int(enable)), "rod_set_tiles")
+
+
+def rod_set_wait_limit(h, polls):
+    _check(load().rod_set_wait_limit(h, int(polls)), "rod_set_wait_limit")
+
+
+def rod_wait_status(h) -> int:
+    """Rods whose tiles lost a wait for a neighbour (their state is NaN) since the last call."""
+    n = ctypes.c_int()
+    _check(load().rod_wait_status(h, ctypes.byref(n)), "rod_wait_status")
+    return n.value
 
 
 KERNEL_KINDS = ("block", "cluster", "grid", "self", "pair", "tiles", "tiles_grid", "pair_tiles")

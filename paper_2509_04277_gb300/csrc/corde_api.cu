@@ -226,6 +226,7 @@ struct corde_rods {
   int last_launches = 0;
   int pdl = 1;  // stepping kernels launched with programmatic stream serialisation
   int tiles = 1;  // warp tiles where they apply (rod_set_tiles)
+  unsigned wait_limit = kTileWaitLimit;  // polls of a tile's wait on a grid (rod_set_wait_limit)
   // rollout / adjoint
   float4* d_ckpt = nullptr;  // [n_ckpt][4][E]
   size_t ckpt_cap = 0;       // float4 entries
@@ -564,6 +565,7 @@ int build_bins(rod_handle h) {
       if (b.tile.per && b.tile.grid) {
         CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
         CK(cudaMemset(b.d_tile_gh, 0, tile_halo_bytes(b.tile.per, nmax)));  // no stamps
+        CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, nmax) + 2, &h->wait_limit, sizeof(unsigned), cudaMemcpyHostToDevice));
         CK(cudaStreamSynchronize(cudaStreamLegacy));  // before a launch on a stream that doesn't wait for this one
       }
     }
@@ -1537,6 +1539,35 @@ int rod_set_tiles(rod_handle h, int enable) {
   free_adjoint_bins(h);  // (built again by the next rod_rollout or rod_adjoint)
   if (int rc = build_bins(h)) return rc;
   return h->pairs.empty() ? CORDE_OK : build_pair_bins(h);
+}
+
+int rod_set_wait_limit(rod_handle h, unsigned polls) {
+  if (int rc = check_handle(h)) return rc;
+  CK(cudaDeviceSynchronize());
+  h->wait_limit = polls;
+  for (const Bin& b : h->bins)
+    if (b.d_tile_gh)
+      CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &polls, sizeof(unsigned), cudaMemcpyHostToDevice));
+  CK(cudaDeviceSynchronize());
+  return CORDE_OK;
+}
+
+int rod_wait_status(rod_handle h, int* n_lost) {
+  if (int rc = check_handle(h)) return rc;
+  if (!n_lost) return fail(CORDE_ERR_ARG, "rod_wait_status: NULL argument");
+  CK(cudaDeviceSynchronize());
+  *n_lost = 0;
+  for (const Bin& b : h->bins) {
+    if (!b.d_tile_gh) continue;
+    unsigned* word = tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 1;
+    unsigned lost = 0;
+    CK(cudaMemcpy(&lost, word, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    if (lost == 0) continue;
+    ++*n_lost;
+    CK(cudaMemset(word, 0, sizeof(unsigned)));
+  }
+  CK(cudaDeviceSynchronize());
+  return CORDE_OK;
 }
 
 int rod_get_kernels(rod_handle h, int* out) {

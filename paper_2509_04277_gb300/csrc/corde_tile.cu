@@ -134,9 +134,22 @@ tile_step_kernel(const RodDev* __restrict__ rods, const int* __restrict__ work, 
 
   // every tile has loaded its ghosts' elements, and read its neighbours' last buffers, before
   // any state is overwritten or any block leaves
+  // (a grid sync has no limit of its own: every block is resident and every wait before it ends)
   if (K > 1) link.barrier();
-  link.leave(k, lane, gh);
-  if (link.lost) rod.spoil();
+  link.leave(k, lane);
+  if constexpr (SYNC == kTileGrid) {
+    // what a wait that ran out let through is anywhere in the rod: nothing of this launch stands
+    if (K > 1 && link.ran_out()) {
+      rod.spoil();
+      if (traj != nullptr && link.owned) {
+        const float nan = __int_as_float(0x7fffffff);
+        for (int step = 0; step < n_steps; ++step)
+#pragma unroll
+          for (int e = 0; e < PER; ++e)
+            if (rod.e0 + e < rod.n) traj[(int64_t)step * n_elem + R.off + rod.e0 + e] = make_float4(nan, nan, nan, rod.w[e]);
+      }
+    }
+  }
   if (link.owned) rod.store(x4, v4, q4, o4, pos_out);
 }
 
@@ -173,7 +186,10 @@ int tile_smem(const TilePlan& p, int warps) {
 int tile_count(int per, int n) { return per == 4 ? Tile<4>::count(n) : Tile<2>::count(n); }
 int64_t tile_halo_bytes(int per, int n) {
   const int64_t buf = per == 4 ? Tile<4>::kGridBuf : Tile<2>::kGridBuf;
-  return (2 * tile_count(per, n) * buf + 1) * (int64_t)sizeof(float4);  // and the last stamp
+  return (2 * tile_count(per, n) * buf + 1) * (int64_t)sizeof(float4);  // and the tail
+}
+unsigned* tile_tail(float4* gh, int per, int n) {
+  return reinterpret_cast<unsigned*>(gh + tile_halo_bytes(per, n) / sizeof(float4) - 1);
 }
 
 cudaError_t prepare_tile(const TilePlan& p) {

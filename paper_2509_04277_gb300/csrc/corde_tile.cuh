@@ -255,7 +255,8 @@ struct TileRod {
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
       const float nan = __int_as_float(0x7fffffff);
-      r[e] = v[e] = f3(nan, nan, nan);
+      r[e] = v[e] = om[e] = f3(nan, nan, nan);
+      q[e] = make_float4(nan, nan, nan, nan);
     }
   }
 
@@ -306,7 +307,9 @@ __device__ __forceinline__ unsigned get_stamped(const float4* p, float& x, float
   z = __uint_as_float(c);
   return stamp;
 }
-constexpr int kTileSpinLimit = 1 << 22;  // polls before a wait for a neighbour gives up (seconds)
+// Behind a grid's exchange buffers: the stamp of its last exchange, the launch in which a wait ran out
+// (launch_id; 0: none), and the polls after which a wait gives up.
+enum TileTail { kTailStamp, kTailLost, kTailLimit };
 
 // A warp's place among the K tiles of a rod (or pair): tile k holds lanes k O ... k O + 31 of it.
 // BUF: float4 of a tile's exchange buffer, of which there are two, used in turn.
@@ -317,9 +320,10 @@ struct TileLink {
   const float4* theirs;     // where a ghost lane's owner publishes (NULL: not a ghost)
   int64_t stride;           // from one buffer to the other
   int parity = 0;
-  // grids: the stamp of the last exchange (it goes on from launch to launch, kept behind the buffers), and
-  // whether a wait has given up
-  unsigned stamp = 0;
+  // grids: the stamp of the last exchange (it goes on from launch to launch, kept behind the buffers); this
+  // launch's id (from the stamp it began with), the polls of a wait, and whether one of the tile's has given up
+  unsigned* tail = nullptr;
+  unsigned stamp = 0, launch_id = 0, limit = 0;
   bool lost = false;
 
   // Q: lanes of the whole rod; smem: the block's buffers, or gh: the grid's
@@ -331,7 +335,12 @@ struct TileLink {
     mine = tile_on_grid(SYNC) ? gh + (int64_t)k * BUF + lane : smem + wid * BUF + lane;
     stride = (int64_t)(tile_on_grid(SYNC) ? K : W) * BUF;
     theirs = nullptr;
-    if constexpr (SYNC == kTileGrid) stamp = __ldcg(reinterpret_cast<const unsigned*>(gh + 2 * stride));
+    if constexpr (SYNC == kTileGrid) {
+      tail = reinterpret_cast<unsigned*>(gh + 2 * stride);
+      stamp = __ldcg(tail + kTailStamp);
+      limit = __ldcg(tail + kTailLimit);
+      launch_id = 2 * stamp + 1;  // (a launch in which a wait can run out moves the stamp)
+    }
     if (active && !owned && g < Q) {
       const int ok = min(max((g - T::G) / T::O, 0), K - 1);  // the tile that owns lane g
       const int ol = g - ok * T::O;
@@ -412,14 +421,22 @@ struct TileLink {
       for (int s = 0; s < M; ++s) put_stamped(m + s * 32, f[3 * s], f[3 * s + 1], f[3 * s + 2], stamp);
     }
     const float4* p = theirs + parity * stride;
-    for (int tries = 0;; ++tries) {
+    for (unsigned tries = 0;; ++tries) {
       unsigned other = 0;
       if (theirs != nullptr) {
 #pragma unroll
         for (int s = 0; s < M; ++s) other |= get_stamped(p + s * 32, f[3 * s], f[3 * s + 1], f[3 * s + 2]) ^ stamp;
       }
       if (__all_sync(0xffffffffu, other == 0)) break;
-      if (lost || tries == kTileSpinLimit) {
+      // A wait that runs out marks the launch, and so ends every other wait: a tile that no longer waits runs ahead,
+      // so its neighbours would each wait for the whole limit, one after the other.
+      if (lost) break;
+      if (tries >= limit) {
+        lost = true;
+        if ((threadIdx.x & 31) == 0) __stcg(tail + kTailLost, launch_id);
+        break;
+      }
+      if ((tries & 255) == 255 && __any_sync(0xffffffffu, ran_out())) {
         lost = true;
         break;
       }
@@ -429,9 +446,11 @@ struct TileLink {
     parity ^= 1;
     return theirs != nullptr;
   }
+  // whether a wait of this launch has run out, on whichever tile (all see it after the launch's last barrier)
+  __device__ __forceinline__ bool ran_out() const { return __ldcg(tail + kTailLost) == launch_id; }
   // after the launch's last barrier: the stamps go on from here
-  __device__ __forceinline__ void leave(int k, int lane, float4* gh) const {
-    if (SYNC == kTileGrid && k == 0 && lane == 0) *reinterpret_cast<unsigned*>(gh + 2 * stride) = stamp;
+  __device__ __forceinline__ void leave(int k, int lane) const {
+    if (SYNC == kTileGrid && k == 0 && lane == 0) tail[kTailStamp] = stamp;
   }
 };
 

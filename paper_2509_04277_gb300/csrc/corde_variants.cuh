@@ -184,6 +184,8 @@ struct TilePlan {
 constexpr int kTileMaxWarps = 8;           // warps per block
 int tile_count(int per, int n);            // tiles (warps) of a rod of n nodes
 int64_t tile_halo_bytes(int per, int n);   // global exchange buffers of a rod on a grid
+constexpr unsigned kTileWaitLimit = 1u << 22;  // polls before a wait for a neighbour gives up (seconds)
+unsigned* tile_tail(float4* gh, int per, int n);  // behind them: words stamp, launch that lost a wait, limit (TileTail)
 int pair_tile_count(int n);                // tiles of a pair of rods of at most n nodes, two elements per lane and rod
 cudaError_t prepare_pair_tile(const TilePlan& p, bool two_way);
 cudaError_t launch_pair_tile(const StepArgs& a, const int4* pairs, int n_pairs, const TilePlan& p, bool two_way,
