@@ -237,8 +237,9 @@ int rod_set_wait_limit(rod_handle h, unsigned polls);
 int rod_wait_status(rod_handle h, int* n_lost);
 
 /* The kernel that steps each rod: out [n_rods][4] ints = one of the kinds below, blocks per rod
- * (or pair), threads per block, elements per thread (per lane on tiles).  With a mailbox
- * enabled, that of a mailbox launch.  Host-side only. */
+ * (or pair), threads per block, elements per thread (per lane on tiles), in a rod_step like the
+ * one before it (see rod_set_graph_mode).  With a mailbox enabled, that of a mailbox launch.
+ * Host-side only. */
 #define CORDE_KERNEL_BLOCK 0       /* one block */
 #define CORDE_KERNEL_CLUSTER 1     /* a cluster of blocks */
 #define CORDE_KERNEL_GRID 2        /* a cooperative grid of blocks */
@@ -283,12 +284,16 @@ int rod_autotune_steps(rod_handle h, const int* candidates, int n_candidates, in
                        void* stream);
 int rod_get_plan(rod_handle h, int* plan);
 
-/* When one rod_step needs several kernel launches (rods of several length bins, bound
- * pairs), rod_step captures them once into a CUDA graph whose kernels run concurrently
- * and replays it (re-captured when n_steps or the plan changes; the drive is first copied
- * into an internal buffer the graph reads).  mode 0: never use a graph; 1: when more than
- * one launch is needed (default); 2: always.  The first rod_step after a change captures
- * on an internal stream: do not call it inside a caller's own stream capture. */
+/* One rod_step takes a kernel launch per plan of the handle's rods (and per layout of its bound
+ * pairs).  mode 0: these launches one after the other, never a graph.  2: always captured into
+ * a CUDA graph whose kernels run concurrently, and replayed (re-captured when n_steps, the
+ * positions output or the plan changes; the drive is first copied into an internal buffer the
+ * graph reads).  1 (default): a rod_step with the n_steps and positions output of the one
+ * before it replays a graph, where its launches are several or the rods fill the GPU and a
+ * plan's are split over blocks of several sizes (rod_last_launch_count then counts more); any
+ * other one launches directly, several launches concurrently on internal streams that the
+ * caller's stream waits for.
+ * Inside a caller's own stream capture the launches are always direct. */
 int rod_set_graph_mode(rod_handle h, int mode);
 
 /* Mailbox of running launches (Section 2.2 and 3.1: the haptic thread writes the device's

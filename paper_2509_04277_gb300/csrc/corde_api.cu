@@ -222,7 +222,11 @@ struct corde_rods {
   std::vector<int> plan;          // variant index per rod (block or cluster table)
   std::vector<int> plan_cluster;  // blocks per rod; 0: one block
   std::vector<char> plan_grid;    // 1: the rod's plan_cluster blocks form a cooperative grid
-  std::vector<Bin> bins;
+  // One launch per bin.  bins: a launch per plan, where launches do not overlap (one stream, a mailbox
+  // whose rods run together, a rollout) or a single one does; graph_bins (empty: the same): split by the
+  // smallest block that holds the rods, for parallel branches of rods that fill the GPU.
+  std::vector<Bin> bins, graph_bins;
+  int* d_work = nullptr;  // the bins' work lists
   int last_launches = 0;
   int pdl = 1;  // stepping kernels launched with programmatic stream serialisation
   int tiles = 1;  // warp tiles where they apply (rod_set_tiles)
@@ -270,6 +274,8 @@ struct corde_rods {
   int graph_steps = -1;
   const float4* graph_drive = nullptr;
   float4* graph_pos_out = nullptr;
+  int last_steps = -1;  // n_steps and positions output of the previous rod_step (-1: changed since)
+  float4* last_pos_out = nullptr;
   float4* io_pos = nullptr;  // positions output of the launch being issued (rod_step_io)
   int graph_launches = 0;
   cudaStream_t cap_stream = nullptr;
@@ -492,12 +498,15 @@ int check_handle(rod_handle h) {
 }
 
 void free_bins(rod_handle h) {
-  for (auto& b : h->bins) {
-    cudaFree(b.d_work);
-    cudaFree(b.d_gh);
-    cudaFree(b.d_tile_gh);
+  for (auto* list : {&h->bins, &h->graph_bins}) {
+    for (auto& b : *list) {
+      cudaFree(b.d_gh);
+      cudaFree(b.d_tile_gh);
+    }
+    list->clear();
   }
-  h->bins.clear();
+  cudaFree(h->d_work);
+  h->d_work = nullptr;
 }
 
 // Group rods by variant; each group's work list is sorted by decreasing length so that
@@ -506,6 +515,7 @@ void invalidate_graph(rod_handle h) {
   if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
   h->graph_exec = nullptr;
   h->graph_steps = -1;
+  h->last_steps = -1;
 }
 
 TileRoom tile_room(rod_handle h) {
@@ -514,20 +524,20 @@ TileRoom tile_room(rod_handle h) {
   return TileRoom{h->sms, h->sms - h->n_rods, warps > 8 * (int64_t)h->sms};
 }
 
-int build_bins(rod_handle h) {
-  invalidate_graph(h);
-  free_bins(h);
-  // Threads of the smallest block that holds the rod in its <4, *> variant.  Power-of-two
-  // blocks are on average 28 % idle warps for log-uniform lengths, which take issue slots in
-  // the constraint sweeps and keep other blocks off the SM.
-  auto trim_of = [&](int r) {
+// The handle's rods in bins of one launch each: by plan, and with by_trim also by the smallest block
+// that holds them.  Nothing is allocated here.
+std::vector<Bin> list_bins(rod_handle h, bool by_trim) {
+  // Threads of the block, in steps of 32 between the powers of two, that a rod's <4, *> variant can shrink
+  // to; 0: none is smaller.  Power-of-two blocks are on average 28 % idle warps for log-uniform lengths,
+  // which take issue slots in the constraint sweeps and keep other blocks off the SM.
+  auto trim_of = [&](int r, int n) {
     if (h->plan_cluster[r] != 0 || variants()[h->plan[r]].ept != 4) return 0;
-    const int t = ((h->n_nodes[r] + 3) / 4 + 31) / 32 * 32;
+    const int t = ((n + 3) / 4 + 31) / 32 * 32;
     return t < variants()[h->plan[r]].nt && trimmed_variant(t) ? t : 0;
   };
   std::vector<std::tuple<int, int, int, int>> keys;  // (blocks per rod, variant, grid, trimmed threads)
   auto key_of = [&](int r) {
-    return std::make_tuple(h->plan_cluster[r], h->plan[r], (int)h->plan_grid[r], trim_of(r));
+    return std::make_tuple(h->plan_cluster[r], h->plan[r], (int)h->plan_grid[r], by_trim ? trim_of(r, h->n_nodes[r]) : 0);
   };
   for (int r = 0; r < h->n_rods; ++r) {
     if (r < (int)h->paired.size() && h->paired[r]) continue;
@@ -536,47 +546,75 @@ int build_bins(rod_handle h) {
   }
   std::sort(keys.begin(), keys.end());
   TileRoom room = tile_room(h);
+  std::vector<Bin> bins;
   for (const auto& k : keys) {
-    std::vector<int> rods;
+    Bin b{std::get<1>(k), 0, nullptr, std::get<0>(k), std::get<2>(k)};
     for (int r = 0; r < h->n_rods; ++r)
-      if (key_of(r) == k && !(r < (int)h->paired.size() && h->paired[r])) rods.push_back(r);
-    // heaviest rods first: a rod's work per step grows with its nodes times (the force
-    // phase, about seven constraint iterations' worth, plus its constraint iterations)
-    std::stable_sort(rods.begin(), rods.end(), [&](int a, int b) {
-      return (int64_t)h->n_nodes[a] * (7 + h->n_iters[a]) > (int64_t)h->n_nodes[b] * (7 + h->n_iters[b]);
+      if (key_of(r) == k && !(r < (int)h->paired.size() && h->paired[r])) b.rods.push_back(r);
+    b.count = (int)b.rods.size();
+    // rods that run longest first (a proxy of a block's step time: nodes x (fixed work +
+    // iterations)), so the tail of the launch overlaps with them
+    std::stable_sort(b.rods.begin(), b.rods.end(), [&](int a, int bb) {
+      return (int64_t)h->n_nodes[a] * (7 + h->n_iters[a]) > (int64_t)h->n_nodes[bb] * (7 + h->n_iters[bb]);
     });
-    Bin b{std::get<1>(k), (int)rods.size(), nullptr, std::get<0>(k), std::get<2>(k)};
-    b.trim = trimmed_variant(std::get<3>(k));
-    b.n_max = 0;
-    for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
-    CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
-    CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
-    b.rods = rods;
-    if (b.grid) {
-      const size_t n4 = rods.size() * 2 * (size_t)b.cluster * kHaloSlots * 2;
-      CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
-      CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
-    }
+    for (int r : b.rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
+    b.trim = trimmed_variant(trim_of(b.rods[0], b.n_max));
     if (b.cluster >= 0 && h->tiles) {
-      const int nmax = b.n_max;
       const int arith = b.cluster > 0 ? kClusterVariants[b.variant].ept : variants()[b.variant].ept;
-      b.tile = tile_plan(nmax, b.count, arith, &room);
+      b.tile = tile_plan(b.n_max, b.count, arith, &room);
+    }
+    bins.push_back(std::move(b));
+  }
+  // the longest rods first: their blocks run longest
+  std::stable_sort(bins.begin(), bins.end(), [](const Bin& a, const Bin& b) { return a.n_max > b.n_max; });
+  return bins;
+}
+
+int alloc_bins(rod_handle h) {
+  h->bins = list_bins(h, false);
+  // Split where the rods fill the GPU: 4096 of 16-2048 nodes 3.98 ms per 100 steps, 4.6 on a launch per plan;
+  // 1000 of 513-1024 1.61 against 1.82.  Rods that leave SMs idle gain nothing (60 of 16-2048 0.57 against 0.55,
+  // 300 of 257-512 0.36 against 0.32) and would pay for the further launches.
+  if (tile_room(h).saturated) h->graph_bins = list_bins(h, true);
+  if (h->graph_bins.size() == h->bins.size()) h->graph_bins.clear();
+  std::vector<int> work;  // the work lists of all bins
+  for (auto* list : {&h->bins, &h->graph_bins})
+    for (const Bin& b : *list) work.insert(work.end(), b.rods.begin(), b.rods.end());
+  if (work.empty()) return CORDE_OK;
+  CK(cudaMalloc(&h->d_work, work.size() * sizeof(int)));
+  CK(cudaMemcpy(h->d_work, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice));
+  int* d = h->d_work;
+  for (auto* list : {&h->bins, &h->graph_bins})
+    for (Bin& b : *list) {
+      b.d_work = d;
+      d += b.count;
+      if (b.grid) {
+        const size_t n4 = (size_t)b.count * 2 * b.cluster * 2 * kHaloSlots;
+        CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
+        CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
+      }
       if (b.tile.per) CK(prepare_tile(b.tile));
       if (b.tile.per && b.tile.grid) {
-        CK(cudaMalloc(&b.d_tile_gh, tile_halo_bytes(b.tile.per, nmax)));
-        CK(cudaMemset(b.d_tile_gh, 0, tile_halo_bytes(b.tile.per, nmax)));  // no stamps
-        CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, nmax) + 2, &h->wait_limit, sizeof(unsigned), cudaMemcpyHostToDevice));
+        const int64_t bytes = tile_halo_bytes(b.tile.per, b.n_max);
+        CK(cudaMalloc(&b.d_tile_gh, bytes));
+        CK(cudaMemset(b.d_tile_gh, 0, bytes));  // no stamps
+        CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &h->wait_limit, sizeof(unsigned),
+                      cudaMemcpyHostToDevice));
         CK(cudaStreamSynchronize(cudaStreamLegacy));  // before a launch on a stream that doesn't wait for this one
       }
     }
-    h->bins.push_back(b);
-  }
-  // the longest rods first: their blocks run longest
-  std::stable_sort(h->bins.begin(), h->bins.end(), [](const Bin& a, const Bin& b) { return a.n_max > b.n_max; });
   return CORDE_OK;
 }
 
-int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* drive, cudaStream_t s,
+int build_bins(rod_handle h) {
+  invalidate_graph(h);
+  free_bins(h);
+  const int rc = alloc_bins(h);
+  if (rc != CORDE_OK) free_bins(h);  // (no bin is left without its device memory)
+  return rc;
+}
+
+int launch_bins(rod_handle h, const Bin* bins, size_t n_bins, int n_steps, const float4* drive, cudaStream_t s,
                 float4* traj = nullptr, const MailboxDev* mb = nullptr, float4* ckpt = nullptr, int ckpt_every = 1) {
   StepArgs a = {};
   a.ckpt = ckpt;
@@ -598,7 +636,8 @@ int launch_bins(rod_handle h, const std::vector<Bin>& bins, int n_steps, const f
   a.pdl = h->pdl;
   if (mb) a.mb = *mb;
   int launches = 0;
-  for (const auto& b : bins) {
+  for (size_t k = 0; k < n_bins; ++k) {
+    const Bin& b = bins[k];
     a.work = b.d_work;
     if (b.tile.per && !mb) {
       a.grid_halo = b.d_tile_gh;
@@ -699,14 +738,12 @@ bool params_valid(const RodParams& p, std::string& why) {
 
 // Launches every bin and pair bin of one rod_step.  With branches, bin k goes to
 // branches[k] (for the forked graph capture); otherwise all go to s in order.
-int launch_all(rod_handle h, int n_steps, const float4* d, cudaStream_t s, const std::vector<cudaStream_t>* branches,
-               const MailboxDev* mb = nullptr) {
+int launch_all(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d, cudaStream_t s,
+               const std::vector<cudaStream_t>* branches, const MailboxDev* mb = nullptr) {
   int launches = 0;
   size_t k = 0;
-  for (size_t b = 0; b < h->bins.size(); ++b, ++k) {
-    cudaStream_t sk = branches ? (*branches)[k] : s;
-    std::vector<Bin> one{h->bins[b]};
-    if (int rc = launch_bins(h, one, n_steps, d, sk, nullptr, mb)) return rc;
+  for (; k < bins.size(); ++k) {
+    if (int rc = launch_bins(h, &bins[k], 1, n_steps, d, branches ? (*branches)[k] : s, nullptr, mb)) return rc;
     ++launches;
   }
   if (!h->pair_bins.empty()) {
@@ -739,12 +776,8 @@ int launch_all(rod_handle h, int n_steps, const float4* d, cudaStream_t s, const
   return CORDE_OK;
 }
 
-// Captures one rod_step into a CUDA graph whose kernel nodes run concurrently (fork on
-// an event, one branch stream per bin, join), so that the bins fill the SMs together.
-int capture_graph(rod_handle h, int n_steps, const float4* d) {
-  invalidate_graph(h);
-  const size_t nb = h->bins.size() + h->pair_bins.size();
-  if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+// Branch streams and events for nb concurrent launches.
+int prepare_fork(rod_handle h, size_t nb) {
   if (!h->fork_ev) CK(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming));
   while (h->side.size() < nb) {
     cudaStream_t st;
@@ -754,15 +787,34 @@ int capture_graph(rod_handle h, int n_steps, const float4* d) {
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     h->join_ev.push_back(ev);
   }
-  CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  return CORDE_OK;
+}
+
+// launch_all on branch streams between a fork from s and a join back to it (also where the launches
+// failed, so that a capture of s can end); *e: a failure of the fork or the join.
+int launch_forked(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d, cudaStream_t s, cudaError_t* e) {
+  const size_t nb = bins.size() + h->pair_bins.size();
   int rc = CORDE_OK;
-  cudaError_t e = cudaEventRecord(h->fork_ev, h->cap_stream);
-  for (size_t k = 0; k < nb && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(h->side[k], h->fork_ev, 0);
-  if (e == cudaSuccess) rc = launch_all(h, n_steps, d, h->cap_stream, &h->side);
-  for (size_t k = 0; k < nb && e == cudaSuccess && rc == CORDE_OK; ++k) {
-    e = cudaEventRecord(h->join_ev[k], h->side[k]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->cap_stream, h->join_ev[k], 0);
+  *e = cudaEventRecord(h->fork_ev, s);
+  for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) *e = cudaStreamWaitEvent(h->side[k], h->fork_ev, 0);
+  if (*e == cudaSuccess) rc = launch_all(h, bins, n_steps, d, s, &h->side);
+  for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) {
+    *e = cudaEventRecord(h->join_ev[k], h->side[k]);
+    if (*e == cudaSuccess) *e = cudaStreamWaitEvent(s, h->join_ev[k], 0);
   }
+  return rc;
+}
+
+// Captures one rod_step into a CUDA graph whose kernel nodes run concurrently (fork on
+// an event, one branch stream per bin, join), so that the bins fill the SMs together.
+int capture_graph(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d) {
+  invalidate_graph(h);
+  const size_t nb = bins.size() + h->pair_bins.size();
+  if (int rc = prepare_fork(h, nb)) return rc;
+  if (!h->cap_stream) CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
+  CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = cudaSuccess;
+  const int rc = launch_forked(h, bins, n_steps, d, h->cap_stream, &e);
   cudaGraph_t g = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
   if (rc != CORDE_OK) {
@@ -950,19 +1002,43 @@ static int step_impl(rod_handle h, int n_steps, const float* drive, float4* pos_
   if (h->mb_period > 0) {
     MailboxDev mb = h->mb_dev;
     mb.step0 = h->steps_done;
-    if (int rc = launch_all(h, n_steps, d, (cudaStream_t)stream, nullptr, &mb)) return rc;
+    if (int rc = launch_all(h, h->bins, n_steps, d, (cudaStream_t)stream, nullptr, &mb)) return rc;
     h->steps_done += n_steps;
     return CORDE_OK;
   }
-  const int n_launch = (int)h->bins.size() + (int)h->pair_bins.size();
-  const bool use_graph = h->graph_mode == 2 || (h->graph_mode == 1 && n_launch > 1);
+  if (h->bins.empty() && h->pair_bins.empty())
+    return fail(CORDE_ERR_CUDA, "rod_step: no launches (an earlier change of the plan failed)");
+  const bool several = h->bins.size() + h->pair_bins.size() > 1;
+  const std::vector<Bin>& gbins = h->graph_mode == 1 && !h->graph_bins.empty() ? h->graph_bins : h->bins;
+  bool use_graph = h->graph_mode == 2 || (h->graph_mode == 1 && (several || !h->graph_bins.empty()));
+  if (use_graph) {
+    // a caller's capture cannot hold a graph launch; and a graph is worth its capture (some 100 us) only
+    // for a step like the one before it
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing((cudaStream_t)stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) use_graph = false;
+    if (h->graph_mode == 1 && (h->last_steps != n_steps || h->last_pos_out != pos_out)) use_graph = false;
+    h->last_steps = n_steps;
+    h->last_pos_out = pos_out;
+  }
   h->steps_done += n_steps;
-  if (!use_graph) return launch_all(h, n_steps, d, (cudaStream_t)stream, nullptr);
+  if (!use_graph) {
+    if (h->graph_mode == 0 || !several) return launch_all(h, h->bins, n_steps, d, (cudaStream_t)stream, nullptr);
+    if (int rc = prepare_fork(h, gbins.size() + h->pair_bins.size())) return rc;
+    const int pdl = h->pdl;
+    h->pdl = 0;  // (a branch starts with an event wait: there is no kernel to overlap with)
+    cudaError_t e = cudaSuccess;
+    const int rc = launch_forked(h, gbins, n_steps, d, (cudaStream_t)stream, &e);
+    h->pdl = pdl;
+    CK(e);
+    return rc;
+  }
   if (!h->d_drive_graph) CK(cudaMalloc(&h->d_drive_graph, h->n_rods * 2 * sizeof(float4)));
   CK(cudaMemcpyAsync(h->d_drive_graph, d, h->n_rods * 2 * sizeof(float4), cudaMemcpyDefault, (cudaStream_t)stream));
   if (!h->graph_exec || h->graph_steps != n_steps || h->graph_drive != h->d_drive_graph ||
       h->graph_pos_out != pos_out) {
-    if (int rc = capture_graph(h, n_steps, h->d_drive_graph)) return rc;
+    if (int rc = capture_graph(h, gbins, n_steps, h->d_drive_graph)) return rc;
+    h->last_steps = n_steps;  // (invalidated with the old graph)
   }
   CK(cudaGraphLaunch(h->graph_exec, (cudaStream_t)stream));
   h->last_launches = h->graph_launches;
@@ -1212,7 +1288,8 @@ int rod_autotune_steps(rod_handle h, const int* candidates, int n_candidates, in
       const int S = candidates[k];
       const int launches = (min_steps + S - 1) / S;
       restore();
-      if ((rc = step_impl(h, S, nullptr, nullptr, s)) != CORDE_OK) break;  // warm-up (and graph capture)
+      for (int w = 0; w < 2 && rc == CORDE_OK; ++w) rc = step_impl(h, S, nullptr, nullptr, s);  // warm-up and graph capture
+      if (rc != CORDE_OK) break;
       restore();
       cudaEventRecord(e0, s);
       for (int l = 0; l < launches && rc == CORDE_OK; ++l) rc = step_impl(h, S, nullptr, nullptr, s);
@@ -1319,18 +1396,18 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         const StepVariant& v = variants()[vi];
         if (v.capacity() < nmax) continue;
         if (v.capacity() >= 8 * nmax && v.nt > 32) continue;  // mostly idle threads
-        std::vector<Bin> one{Bin{(int)vi, (int)rods.size(), d_work}};
+        std::vector<Bin> one(1, Bin{(int)vi, (int)rods.size(), d_work});
         TileRoom room = tile_room(h);
         if (h->tiles) one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
         if (one[0].tile.per && prepare_tile(one[0].tile) != cudaSuccess) one[0].tile.per = 0;
         restore();
-        if ((rc = launch_bins(h, one, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
+        if ((rc = launch_bins(h, one.data(), 1, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
         float best_rep = 1e30f;
         for (int rep = 0; rep < 3; ++rep) {
           float ms = 0.f;
           restore();
           cudaEventRecord(e0, s);
-          if ((rc = launch_bins(h, one, n_steps, h->d_drive, s)) != CORDE_OK) break;
+          if ((rc = launch_bins(h, one.data(), 1, n_steps, h->d_drive, s)) != CORDE_OK) break;
           cudaEventRecord(e1, s);
           if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(CORDE_ERR_CUDA, "autotune timing"); break; }
           cudaEventElapsedTime(&ms, e0, e1);
@@ -1545,9 +1622,10 @@ int rod_set_wait_limit(rod_handle h, unsigned polls) {
   if (int rc = check_handle(h)) return rc;
   CK(cudaDeviceSynchronize());
   h->wait_limit = polls;
-  for (const Bin& b : h->bins)
-    if (b.d_tile_gh)
-      CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &polls, sizeof(unsigned), cudaMemcpyHostToDevice));
+  for (auto* list : {&h->bins, &h->graph_bins})
+    for (const Bin& b : *list)
+      if (b.d_tile_gh)
+        CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &polls, sizeof(unsigned), cudaMemcpyHostToDevice));
   CK(cudaDeviceSynchronize());
   return CORDE_OK;
 }
@@ -1557,7 +1635,7 @@ int rod_wait_status(rod_handle h, int* n_lost) {
   if (!n_lost) return fail(CORDE_ERR_ARG, "rod_wait_status: NULL argument");
   CK(cudaDeviceSynchronize());
   *n_lost = 0;
-  for (const Bin& b : h->bins) {
+  for (auto* list : {&h->bins, &h->graph_bins}) for (const Bin& b : *list) {
     if (!b.d_tile_gh) continue;
     unsigned* word = tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 1;
     unsigned lost = 0;
@@ -1576,8 +1654,8 @@ int rod_get_kernels(rod_handle h, int* out) {
     const int k[4] = {kind, blocks, threads, per};
     std::copy(k, k + 4, out + 4 * r);
   };
-  const bool tiles = h->mb_period == 0;
-  for (const Bin& b : h->bins)
+  const bool tiles = h->mb_period == 0, graph = tiles && h->graph_mode == 1 && !h->graph_bins.empty();
+  for (const Bin& b : graph ? h->graph_bins : h->bins)
     for (int r : b.rods) {
       if (b.tile.per && tiles) {
         put(r, b.tile.grid ? CORDE_KERNEL_TILES_GRID : CORDE_KERNEL_TILES, b.tile.blocks, 32 * b.tile.warps, b.tile.per);
@@ -1663,7 +1741,8 @@ int rod_rollout(rod_handle h, int n_steps, int ckpt_every, float* pos_traj, void
   const std::vector<Bin>& bins = adj ? h->adj_bins : h->bins;
   int launches = 0;
   if (adj) {  // all segments in one launch per bin
-    if (int rc = launch_bins(h, bins, n_steps, h->d_drive, s, traj, nullptr, h->d_ckpt, ckpt_every)) return rc;
+    if (int rc = launch_bins(h, bins.data(), bins.size(), n_steps, h->d_drive, s, traj, nullptr, h->d_ckpt, ckpt_every))
+      return rc;
     launches = h->last_launches;
   }
   for (int seg = 0; seg < n_seg && !adj; ++seg) {
@@ -1672,7 +1751,8 @@ int rod_rollout(rod_handle h, int n_steps, int ckpt_every, float* pos_traj, void
     CK(launch_copy4(c, E, 0, s));
     const int t0 = seg * ckpt_every;
     const int cnt = std::min(ckpt_every, n_steps - t0);
-    if (int rc = launch_bins(h, bins, cnt, h->d_drive, s, traj ? traj + (size_t)t0 * E : nullptr)) return rc;
+    if (int rc = launch_bins(h, bins.data(), bins.size(), cnt, h->d_drive, s, traj ? traj + (size_t)t0 * E : nullptr))
+      return rc;
     launches += h->last_launches;
   }
   h->last_launches = launches;
