@@ -173,6 +173,10 @@ struct TileRoom {
 //    with more than eight warps per SM so do single tiles of four elements per lane (4864 of 128: 11.1 / 10.0).
 //  - A rod of one tile of two elements per lane repeats nothing: shuffles beat shared memory at any
 //    load, with the registers of 16 warps per SM (4864 rods of 64 nodes 5.08 us/step against 5.42).
+//  - A plan's clusters all run at once.  Where the device holds fewer of them than there are rods (a cluster of 9
+//    to 16 blocks needs as many free SMs of one GPC; 7 of 16 blocks x 7 warps), four elements per lane take half
+//    the blocks (8 rods of 2048 nodes: 3.42 us/step, 4.79 in two waves), or the plan's kernel runs (8 of
+//    10000: 6.70, 7.38 in two waves).
 TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   TilePlan p;
   p.arith = arith;
@@ -189,8 +193,20 @@ TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   p.full = p.grid && p.warps > kTileMaxWarps;  // up to 16 warps on every SM
   const int64_t more = (int64_t)(p.blocks - 1) * count;
   if (p.blocks >= 1 && p.warps <= (p.full ? 2 : 1) * kTileMaxWarps && !(p.grid && count > 1) && room->spare >= more) {
-    room->spare -= (int)more;
-    return p;
+    bool fits = prepare_tile(p) >= count;
+    for (int most : {kMaxCluster, 8}) {
+      if (fits || p.grid) break;
+      const int blocks = std::min((K4 + 3) / 4, most);
+      if (K4 > kTileMaxWarps * blocks || blocks >= p.blocks) continue;
+      p.per = 4;
+      p.blocks = blocks;
+      p.warps = (K4 + blocks - 1) / blocks;
+      fits = prepare_tile(p) >= count;
+    }
+    if (fits) {
+      room->spare -= (p.blocks - 1) * count;
+      return p;
+    }
   }
   p.grid = 0;
   p.blocks = 1;
@@ -198,6 +214,7 @@ TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   p.warps = K2 == 1 ? 1 : K4;
   p.full = K2 == 1;
   if (!p.full && (room->saturated || K4 > 4 || count > 8 / K4 * room->sms)) p.per = 0;
+  if (p.per && prepare_tile(p) == 0) p.per = 0;
   return p;
 }
 
@@ -593,7 +610,6 @@ int alloc_bins(rod_handle h) {
         CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
         CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
       }
-      if (b.tile.per) CK(prepare_tile(b.tile));
       if (b.tile.per && b.tile.grid) {
         const int64_t bytes = tile_halo_bytes(b.tile.per, b.n_max);
         CK(cudaMalloc(&b.d_tile_gh, bytes));
@@ -1399,7 +1415,6 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         std::vector<Bin> one(1, Bin{(int)vi, (int)rods.size(), d_work});
         TileRoom room = tile_room(h);
         if (h->tiles) one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
-        if (one[0].tile.per && prepare_tile(one[0].tile) != cudaSuccess) one[0].tile.per = 0;
         restore();
         if ((rc = launch_bins(h, one.data(), 1, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
         float best_rep = 1e30f;
@@ -1564,17 +1579,25 @@ static int build_pair_bins(rod_handle h) {
       if (ps.empty()) continue;
       corde_rods::PairBin pb{ept, nt, (int)ps.size(), nullptr, false, TilePlan()};
       for (const int4& p : ps) pb.two_way |= p.z == 2;
-      // tiles of both rods while they find idle SMs (see tile_plan): four warps per block, up to
-      // eight over the largest cluster
+      // tiles of both rods while they find idle SMs (see tile_plan): four warps per block, up to eight over
+      // the largest cluster.  Each bin is held against the whole GPU: beside other bins' tiles it shares SMs, two
+      // blocks each, and still wins (6 pairs of 512 and 6 of 700 nodes 10.3 us/step, 24.2 with one of the bins as
+      // blocks; 8 pairs of 512 and 3 rods of 10000 6.2, 7.2).  Clusters that the device does not hold all at once run in
+      // waves: two still beat the four-element block kernel (8 pairs of 1024 nodes 11.1 us/step, 27.6 as
+      // blocks), not the two-element one (512 nodes: 4.2 a wave, 8.65), whose pairs then take eight blocks a
+      // cluster (11 pairs: 5.3).
       int n_max = 0;
       for (const int4& p : ps) n_max = std::max({n_max, h->n_nodes[p.x], h->n_nodes[p.y]});
       const int K = pair_tile_count(n_max);
       pb.tile.arith = ept;
-      pb.tile.blocks = std::min((K + 3) / 4, kMaxCluster);
-      pb.tile.warps = (K + pb.tile.blocks - 1) / pb.tile.blocks;
-      if (h->tiles && pb.tile.warps <= kTileMaxWarps && (int64_t)pb.tile.blocks * pb.count + h->n_rods <= h->sms) {
-        CK(prepare_pair_tile(pb.tile, pb.two_way));
-        pb.tile.per = 2;
+      for (int most : {kMaxCluster, 8}) {
+        pb.tile.blocks = std::min((K + 3) / 4, most);
+        pb.tile.warps = (K + pb.tile.blocks - 1) / pb.tile.blocks;
+        if (h->tiles && pb.tile.warps <= kTileMaxWarps && (int64_t)pb.tile.blocks * pb.count + h->n_rods <= h->sms &&
+            (int64_t)(ept == 4 ? 2 : 1) * prepare_pair_tile(pb.tile, pb.two_way) >= pb.count) {
+          pb.tile.per = 2;
+          break;
+        }
       }
       CK(cudaMalloc(&pb.d_pairs, ps.size() * sizeof(int4)));
       CK(cudaMemcpy(pb.d_pairs, ps.data(), ps.size() * sizeof(int4), cudaMemcpyHostToDevice));
@@ -1706,7 +1729,6 @@ static int build_adjoint_bins(rod_handle h) {
     // two or more tiles in one block don't pay here: a training step of 256 rods of 256 nodes took
     // 2.77 ms against 2.65 with the block kernel, though the rollout alone is no slower
     if (b.tile.blocks == 1 && b.tile.warps > 1 && b.count > h->sms) b.tile.per = 0;
-    if (b.tile.per) CK(prepare_tile(b.tile));
     h->adj_bins.push_back(b);
   }
   return CORDE_OK;

@@ -201,12 +201,10 @@ static PairTileFn pair_tile_fn(const TilePlan& p, bool two_way) {
   return two_way ? pair_tile_kernel<2, true> : pair_tile_kernel<2, false>;
 }
 
-cudaError_t prepare_pair_tile(const TilePlan& p, bool two_way) {
-  const PairTileFn fn = pair_tile_fn(p, two_way);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       2 * kTileMaxWarps * kPairBuf * (int)sizeof(float4));
-  if (e == cudaSuccess && p.blocks > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e;
+int prepare_pair_tile(const TilePlan& p, bool two_way) {
+  constexpr int kWarpSmem = 2 * kPairBuf * (int)sizeof(float4);
+  return prepare_cluster(reinterpret_cast<const void*>(pair_tile_fn(p, two_way)), p, kTileMaxWarps * kWarpSmem,
+                         p.warps * kWarpSmem);
 }
 
 cudaError_t launch_pair_tile(const StepArgs& a, const int4* pairs, int n_pairs, const TilePlan& p, bool two_way,

@@ -14,6 +14,8 @@
 // the same order (ARITH elements per thread there: the layout decides the order in which
 // an element's force contributions are added and the form of the impulses), so the results
 // are the same bit for bit, whichever kernel runs.
+#include <climits>
+
 #include "corde_tile.cuh"
 
 namespace corde {
@@ -183,6 +185,28 @@ int tile_smem(const TilePlan& p, int warps) {
 
 }  // namespace
 
+int prepare_cluster(const void* fn, const TilePlan& p, int smem_max, int smem) {
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+  if (e == cudaSuccess && p.blocks > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  int n = INT_MAX;
+  if (e == cudaSuccess && p.blocks > 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.blocks);
+    cfg.blockDim = dim3(32 * p.warps);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = p.blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+  }
+  if (e == cudaSuccess) return n;
+  cudaGetLastError();
+  return 0;
+}
+
 int tile_count(int per, int n) { return per == 4 ? Tile<4>::count(n) : Tile<2>::count(n); }
 int64_t tile_halo_bytes(int per, int n) {
   const int64_t buf = per == 4 ? Tile<4>::kGridBuf : Tile<2>::kGridBuf;
@@ -192,14 +216,13 @@ unsigned* tile_tail(float4* gh, int per, int n) {
   return reinterpret_cast<unsigned*>(gh + tile_halo_bytes(per, n) / sizeof(float4) - 1);
 }
 
-cudaError_t prepare_tile(const TilePlan& p) {
+int prepare_tile(const TilePlan& p) {
   const TileFn fn = tile_fn(p);
-  if (fn == nullptr) return cudaErrorInvalidValue;
-  cudaError_t e = cudaSuccess;
-  if (!p.grid) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem(p, kTileMaxWarps));
-  if (e == cudaSuccess && p.blocks > 8 && !p.grid)
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e;
+  if (fn == nullptr) return 0;
+  if (!p.grid) return prepare_cluster(reinterpret_cast<const void*>(fn), p, tile_smem(p, kTileMaxWarps), tile_smem(p, p.warps));
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * p.warps, 0) != cudaSuccess) cudaGetLastError();
+  return per_sm > 0 ? 1 : 0;  // (a block per SM: the plan has no more)
 }
 
 cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s) {

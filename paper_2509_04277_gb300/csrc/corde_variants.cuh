@@ -187,10 +187,13 @@ int64_t tile_halo_bytes(int per, int n);   // global exchange buffers of a rod o
 constexpr unsigned kTileWaitLimit = 1u << 22;  // polls before a wait for a neighbour gives up (seconds)
 unsigned* tile_tail(float4* gh, int per, int n);  // behind them: words stamp, launch that lost a wait, limit (TileTail)
 int pair_tile_count(int n);                // tiles of a pair of rods of at most n nodes, two elements per lane and rod
-cudaError_t prepare_pair_tile(const TilePlan& p, bool two_way);
+// Kernel attributes of the plan's launches on the current device, and how many of the plan's clusters (or grids) it
+// holds at once: 0 if it can't launch them (a cluster of 9 to 16 blocks needs as many SMs of one GPC).
+int prepare_tile(const TilePlan& p);
+int prepare_pair_tile(const TilePlan& p, bool two_way);
+int prepare_cluster(const void* fn, const TilePlan& p, int smem_max, int smem);  // the same for one kernel
 cudaError_t launch_pair_tile(const StepArgs& a, const int4* pairs, int n_pairs, const TilePlan& p, bool two_way,
                              cudaStream_t s);
-cudaError_t prepare_tile(const TilePlan& p);  // kernel attributes of the plan's launches, on the current device
 cudaError_t launch_tile(const StepArgs& a, int n_rods, const TilePlan& p, cudaStream_t s);
 
 // Defined in the per-EPT instantiation units.
