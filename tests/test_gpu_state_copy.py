@@ -50,3 +50,30 @@ def test_device_buffers(corde, n, shift, given):
             want = np.concatenate([want[:, :3], host[k][:, 3:]], axis=1)
         assert np.array_equal(after[k], want)
     b.close()
+
+
+# one element per thread up to 65536, four above; the arrays not given leave no gap
+@pytest.mark.parametrize("given", [(1, 1, 1, 1), (1, 0, 1, 0), (0, 1, 0, 1), (0, 0, 1, 0)])
+@pytest.mark.parametrize("extra", [None, 2, 3, 1027])
+def test_many_elements(corde, extra, given):
+    import torch
+
+    rods = [W.guidewire(512, seed=1)] * 128 + ([W.guidewire(extra, seed=2)] if extra else [])
+    b = corde.RodBatch(rods)
+    b.step(2)
+    host, E = b.state_numpy(), b.n_elem
+    out = [torch.full((E + 1, 4), -7.0, device="cuda") for _ in KEYS]
+    corde.rod_get_state(b.handle, *[o if g else None for o, g in zip(out, given)])
+    for o, g, k in zip(out, given, KEYS):
+        got = o.cpu().numpy()
+        assert np.array_equal(got[:E], host[k] if g else np.full((E, 4), -7.0, np.float32)), k
+        assert (got[E] == -7.0).all()
+    new = [torch.rand((E, 4), device="cuda") for _ in KEYS]
+    corde.rod_set_state(b.handle, *[t if g else None for t, g in zip(new, given)])
+    after = b.state_numpy()
+    for t, g, k in zip(new, given, KEYS):
+        want = t.cpu().numpy() if g else host[k]
+        if k == "pos4":
+            want = np.concatenate([want[:, :3], host[k][:, 3:]], axis=1)
+        assert np.array_equal(after[k], want), k
+    b.close()
