@@ -1,5 +1,7 @@
 // C ABI of the CoRdE stepper: creation (derived constants and packing on the device),
 // kernel-variant plans, the persistent step launches, state I/O and diagnostics.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -521,15 +523,49 @@ cudaError_t launch_copy4(const Copy4& c, int64_t n, int keep_w, cudaStream_t s) 
   return cudaGetLastError();
 }
 
-// True if p (or NULL) is memory of device `dev`, 16-byte aligned: copy4_kernel may use it.
-bool on_device(const void* p, int dev) {
-  if (p == nullptr) return true;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// What copy4_kernel may do with n float4 at p: 1: p (or NULL) is memory of device `dev`, 16-byte aligned, and
+// holds them; 0: not such memory, the copy is cudaMemcpyAsync's; -1: such memory, but it ends before (which
+// cudaMemcpyAsync refuses, and a kernel would not notice).
+int on_device(const void* p, int64_t n, int dev) {
+  if (p == nullptr) return 1;
+  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    return cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) == cudaSuccess &&
+                   found == cudaDriverEntryPointSuccess
+               ? reinterpret_cast<Query>(f)
+               : nullptr;
+  }();
+  if (query == nullptr || reinterpret_cast<uintptr_t>(p) % 16 != 0) return 0;
+  const CUdeviceptr end = reinterpret_cast<CUdeviceptr>(p) + (CUdeviceptr)n * sizeof(float4);
+  // (memory mapped in pieces is a range per piece; one allocation's neighbour is not part of it)
+  for (CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p); at < end;) {
+    unsigned type = 0, managed = 0, whole = 0;
+    int ordinal = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
+    void* out[] = {&type, &managed, &ordinal, &start, &size, &whole};
+    const bool device = query(6, what, out, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && !managed &&
+                        ordinal == dev && start + size > at;
+    if (!device) return at == reinterpret_cast<CUdeviceptr>(p) ? 0 : -1;
+    at = start + size;
+    if (whole && at < end) return -1;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+  return 1;
+}
+// The same of four arrays: -1 if one ends too early, 0 if one is not such memory.
+int all_on_device(const void* const (&p)[4], int64_t n, int dev) {
+  int ok = 1;
+  for (const void* q : p) {
+    const int k = on_device(q, n, dev);
+    if (k < 0) return k;
+    ok = std::min(ok, k);
+  }
+  return ok;
 }
 
 int check_handle(rod_handle h) {
@@ -1116,8 +1152,9 @@ int rod_get_state(rod_handle h, float* pos4, float* quat4, float* vel4, float* o
   if (int rc = check_handle(h)) return rc;
   const size_t b = (size_t)h->n_elem * sizeof(float4);
   cudaStream_t s = (cudaStream_t)stream;
-  if (on_device(pos4, h->device) && on_device(quat4, h->device) && on_device(vel4, h->device) &&
-      on_device(omega4, h->device)) {
+  const int dev = all_on_device({pos4, quat4, vel4, omega4}, h->n_elem, h->device);
+  if (dev < 0) return fail(CORDE_ERR_CUDA, "rod_get_state: a device buffer is shorter than the handle's elements");
+  if (dev) {
     Copy4 c = {{pos4 ? h->d_x : nullptr, quat4 ? h->d_q : nullptr, vel4 ? h->d_v : nullptr, omega4 ? h->d_o : nullptr},
                {(float4*)pos4, (float4*)quat4, (float4*)vel4, (float4*)omega4}};
     CK(launch_copy4(c, h->n_elem, 0, s));
@@ -1135,8 +1172,9 @@ int rod_set_state(rod_handle h, const float* pos4, const float* quat4, const flo
   if (int rc = check_handle(h)) return rc;
   const size_t b = (size_t)h->n_elem * sizeof(float4);
   cudaStream_t s = (cudaStream_t)stream;
-  if (on_device(pos4, h->device) && on_device(quat4, h->device) && on_device(vel4, h->device) &&
-      on_device(omega4, h->device)) {
+  const int dev = all_on_device({pos4, quat4, vel4, omega4}, h->n_elem, h->device);
+  if (dev < 0) return fail(CORDE_ERR_CUDA, "rod_set_state: a device buffer is shorter than the handle's elements");
+  if (dev) {
     Copy4 c = {{(const float4*)pos4, (const float4*)quat4, (const float4*)vel4, (const float4*)omega4},
                {h->d_x, h->d_q, h->d_v, h->d_o}};
     CK(launch_copy4(c, h->n_elem, 1, s));

@@ -77,3 +77,32 @@ def test_many_elements(corde, extra, given):
             want = np.concatenate([want[:, :3], host[k][:, 3:]], axis=1)
         assert np.array_equal(after[k], want), k
     b.close()
+
+
+@pytest.mark.parametrize("which", [0, 2])
+def test_buffer_that_ends_too_early(corde, which):
+    """A device buffer up to the end of its allocation serves; one that is shorter is refused on the host."""
+    import torch
+
+    E = 65536
+    b = corde.RodBatch([W.guidewire(512, seed=1)] * 128)
+    # torch hands allocations above 10 MB out whole, in multiples of 2 MB
+    big = torch.empty(32 << 20, dtype=torch.uint8, device="cuda")
+    assert big.untyped_storage().nbytes() % (2 << 20) == 0
+    rest = [torch.zeros((E, 4), device="cuda") for _ in KEYS]
+
+    def given(spare):
+        args = list(rest)
+        args[which] = big.data_ptr() + big.numel() - 16 * (E - spare)
+        return args
+
+    corde.rod_get_state(b.handle, *given(0))
+    want = b.state_numpy()[KEYS[which]]
+    assert np.array_equal(big[-16 * E:].view(torch.float32).cpu().numpy().reshape(E, 4), want)
+    corde.rod_set_state(b.handle, *given(0))
+    for spare in (1, E // 2):
+        for call in (corde.rod_get_state, corde.rod_set_state):
+            with pytest.raises(corde.CordeError):
+                call(b.handle, *given(spare))
+    torch.cuda.synchronize()
+    b.close()
