@@ -211,8 +211,10 @@ int rod_diagnostics(rod_handle h, double* out);
  * multi-block kernel, Section 2.2).  rod_set_plan forces one block variant for every rod
  * it can hold (ept = 0 restores the default plan); rod_set_plan_cluster forces a cluster
  * variant (ept, nt) in {(2,256), (4,256), (4,512)}, cluster 2..16, for every rod it can
- * hold; rod_autotune times the block variants that hold each length bin on the current
- * state (saved and restored) and keeps the fastest per bin.  rod_get_plan writes
+ * hold; rod_autotune times the block variants that hold each length class on the current
+ * state (saved and restored), with the block sizes they run with, and keeps the fastest per
+ * class; where the class would run on warp tiles and no mailbox is enabled, the tiles of the
+ * fastest variant of each ept decide between the two, unless within 5 %.  rod_get_plan writes
  * [n_rods][3] ints (ept, nt, blocks; 0 = one block, C >= 2 a cluster of C blocks, -C a
  * cooperative grid of C blocks, see rod_set_plan_grid).  Synchronous.
  * A plan fixes the arithmetic: the order in which an element's contributions are added and

@@ -816,14 +816,14 @@ bool params_valid(const RodParams& p, std::string& why) {
 // Launches every bin and pair bin of one rod_step.  With branches, bin k goes to
 // branches[k] (for the forked graph capture); otherwise all go to s in order.
 int launch_all(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d, cudaStream_t s,
-               const std::vector<cudaStream_t>* branches, const MailboxDev* mb = nullptr) {
+               const std::vector<cudaStream_t>* branches, const MailboxDev* mb = nullptr, bool pairs = true) {
   int launches = 0;
   size_t k = 0;
   for (; k < bins.size(); ++k) {
     if (int rc = launch_bins(h, &bins[k], 1, n_steps, d, branches ? (*branches)[k] : s, nullptr, mb)) return rc;
     ++launches;
   }
-  if (!h->pair_bins.empty()) {
+  if (pairs && !h->pair_bins.empty()) {
     StepArgs a = {};
     a.rods = h->d_rods;
     a.work = nullptr;
@@ -869,12 +869,16 @@ int prepare_fork(rod_handle h, size_t nb) {
 
 // launch_all on branch streams between a fork from s and a join back to it (also where the launches
 // failed, so that a capture of s can end); *e: a failure of the fork or the join.
-int launch_forked(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d, cudaStream_t s, cudaError_t* e) {
-  const size_t nb = bins.size() + h->pair_bins.size();
+int launch_forked(rod_handle h, const std::vector<Bin>& bins, int n_steps, const float4* d, cudaStream_t s, cudaError_t* e,
+                  bool pairs = true) {
+  const size_t nb = bins.size() + (pairs ? h->pair_bins.size() : 0);
   int rc = CORDE_OK;
   *e = cudaEventRecord(h->fork_ev, s);
   for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) *e = cudaStreamWaitEvent(h->side[k], h->fork_ev, 0);
-  if (*e == cudaSuccess) rc = launch_all(h, bins, n_steps, d, s, &h->side);
+  const int pdl = h->pdl;
+  if (s != h->cap_stream) h->pdl = 0;  // (a branch starts with an event wait: there is no kernel to overlap with)
+  if (*e == cudaSuccess) rc = launch_all(h, bins, n_steps, d, s, &h->side, nullptr, pairs);
+  h->pdl = pdl;
   for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) {
     *e = cudaEventRecord(h->join_ev[k], h->side[k]);
     if (*e == cudaSuccess) *e = cudaStreamWaitEvent(s, h->join_ev[k], 0);
@@ -1102,11 +1106,8 @@ static int step_impl(rod_handle h, int n_steps, const float* drive, float4* pos_
   if (!use_graph) {
     if (h->graph_mode == 0 || !several) return launch_all(h, h->bins, n_steps, d, (cudaStream_t)stream, nullptr);
     if (int rc = prepare_fork(h, gbins.size() + h->pair_bins.size())) return rc;
-    const int pdl = h->pdl;
-    h->pdl = 0;  // (a branch starts with an event wait: there is no kernel to overlap with)
     cudaError_t e = cudaSuccess;
     const int rc = launch_forked(h, gbins, n_steps, d, (cudaStream_t)stream, &e);
-    h->pdl = pdl;
     CK(e);
     return rc;
   }
@@ -1457,46 +1458,94 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         nmax = std::max(nmax, h->n_nodes[r]);
       }
     if (rods.empty()) continue;
-    std::stable_sort(rods.begin(), rods.end(), [&](int a, int bb) {
-      return (int64_t)h->n_nodes[a] * (7 + h->n_iters[a]) > (int64_t)h->n_nodes[bb] * (7 + h->n_iters[bb]);
-    });
     int* d_work = nullptr;
     if (cudaMalloc(&d_work, rods.size() * sizeof(int)) != cudaSuccess) { rc = fail(CORDE_ERR_OOM, "autotune work list"); break; }
-    cudaMemcpy(d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice);
-    float best_ms = 1e30f;
-    int best_v = -1;
-    // Each candidate: one warm-up launch, then the best of three timed launches from the same
-    // state.  The whole sweep runs twice and only the second pass counts, so that the first
+    const std::vector<int> kept = h->plan;
+    // The class's launches under variant vi: its rods of the bins that the whole handle would have, so with the
+    // trimmed blocks and the share of the room for tiles that they will run with.
+    auto trial = [&](int vi) {
+      for (int r : rods) h->plan[r] = vi;
+      std::vector<Bin> bins = list_bins(h, tile_room(h).saturated), mine;
+      std::vector<int> work;
+      for (Bin& b : bins) {
+        std::vector<int> in;
+        for (int r : b.rods)
+          if (cls[r] == c) in.push_back(r);
+        if (in.empty() || b.cluster != 0) continue;
+        b.rods = in;
+        b.count = (int)in.size();
+        b.d_work = d_work + work.size();
+        work.insert(work.end(), in.begin(), in.end());
+        mine.push_back(b);
+      }
+      h->plan = kept;
+      cudaMemcpy(d_work, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice);
+      return mine;
+    };
+    auto run = [&](const std::vector<Bin>& bins) {
+      if (bins.size() == 1) return launch_bins(h, bins.data(), 1, n_steps, h->d_drive, s);
+      if (int e = prepare_fork(h, bins.size())) return e;
+      cudaError_t e = cudaSuccess;
+      const int r = launch_forked(h, bins, n_steps, h->d_drive, s, &e, false);
+      return r == CORDE_OK && e != cudaSuccess ? fail(CORDE_ERR_CUDA, "autotune launches") : r;
+    };
+    // One warm-up launch, then the best of three timed launches from the same state.
+    auto best_of = [&](const std::vector<Bin>& bins, float* best) {
+      restore();
+      if (int e = run(bins)) return e;
+      *best = 1e30f;
+      for (int rep = 0; rep < 3; ++rep) {
+        float ms = 0.f;
+        restore();
+        cudaEventRecord(e0, s);
+        if (int e = run(bins)) return e;
+        cudaEventRecord(e1, s);
+        if (cudaEventSynchronize(e1) != cudaSuccess) return fail(CORDE_ERR_CUDA, "autotune timing");
+        cudaEventElapsedTime(&ms, e0, e1);
+        *best = std::min(*best, ms);
+      }
+      return (int)CORDE_OK;
+    };
+    // Block variants: the fastest of each ept (nt is what runs under a mailbox or without room for tiles).  Then
+    // between the two, by the tiles where they would run and the block elsewhere; within 5 %, by the blocks: tiles of
+    // both layouts differ by little.  The whole sweep runs twice and only the second pass counts, so that the first
     // candidates are not measured while the clocks still ramp up from idle.
+    int best_v = -1;
     for (int pass = 0; pass < 2 && rc == CORDE_OK; ++pass) {
-      best_ms = 1e30f;
-      best_v = -1;
-      for (size_t vi = 0; vi < variants().size(); ++vi) {
+      struct Best {
+        int v = -1;
+        float block = 1e30f, ms = 1e30f;
+      } best[2];
+      std::vector<std::pair<int, std::vector<int>>> seen;  // (ept, threads of the launches): a larger nt may trim to the same
+      for (size_t vi = 0; vi < variants().size() && rc == CORDE_OK; ++vi) {
         const StepVariant& v = variants()[vi];
         if (v.capacity() < nmax) continue;
         if (v.capacity() >= 8 * nmax && v.nt > 32) continue;  // mostly idle threads
-        std::vector<Bin> one(1, Bin{(int)vi, (int)rods.size(), d_work});
-        TileRoom room = tile_room(h);
-        if (h->tiles) one[0].tile = tile_plan(nmax, (int)rods.size(), v.ept, &room);
-        restore();
-        if ((rc = launch_bins(h, one.data(), 1, n_steps, h->d_drive, s)) != CORDE_OK) break;  // warm-up
-        float best_rep = 1e30f;
-        for (int rep = 0; rep < 3; ++rep) {
-          float ms = 0.f;
-          restore();
-          cudaEventRecord(e0, s);
-          if ((rc = launch_bins(h, one.data(), 1, n_steps, h->d_drive, s)) != CORDE_OK) break;
-          cudaEventRecord(e1, s);
-          if (cudaEventSynchronize(e1) != cudaSuccess) { rc = fail(CORDE_ERR_CUDA, "autotune timing"); break; }
-          cudaEventElapsedTime(&ms, e0, e1);
-          best_rep = std::min(best_rep, ms);
+        std::vector<Bin> bins = trial((int)vi);
+        std::pair<int, std::vector<int>> sig(v.ept, {});
+        for (Bin& b : bins) {
+          b.tile.per = 0;
+          sig.second.push_back(b.trim ? b.trim->nt : v.nt);
         }
-        if (rc != CORDE_OK) break;
-        if (best_rep < best_ms) { best_ms = best_rep; best_v = (int)vi; }
+        if (std::find(seen.begin(), seen.end(), sig) != seen.end()) continue;
+        seen.push_back(sig);
+        float ms = 0.f;
+        if ((rc = best_of(bins, &ms)) != CORDE_OK) break;
+        Best& be = best[v.ept == 4];
+        if (ms < be.block) be.v = (int)vi, be.block = be.ms = ms;
       }
+      for (Best& be : best) {
+        if (rc != CORDE_OK || be.v < 0 || h->mb_period > 0) continue;
+        const std::vector<Bin> bins = trial(be.v);
+        bool tiles = false;
+        for (const Bin& b : bins) tiles |= b.tile.per > 0;
+        if (tiles) rc = best_of(bins, &be.ms);
+      }
+      const bool tie = std::max(best[0].ms, best[1].ms) < 1.05f * std::min(best[0].ms, best[1].ms);
+      best_v = (tie ? best[1].block < best[0].block : best[1].ms < best[0].ms) ? best[1].v : best[0].v;
     }
     cudaFree(d_work);
-    if (best_v >= 0)
+    if (rc == CORDE_OK && best_v >= 0)
       for (int r : rods) h->plan[r] = best_v;
   }
   restore();
