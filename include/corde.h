@@ -439,7 +439,8 @@ int rod_set_adjoint_record_budget(rod_handle h, long long bytes);
  * Tiles: with at most 10 constraint iterations, every step's records and states within the
  * record budget (per step and node 2 n_iters x 12 B and 64 B) and a block per four tiles of
  * every rod finding an SM of its own (a rod of n nodes has about n / 20 tiles), all checkpoint
- * segments are recorded at once and reversed on overlapping warp tiles.
+ * segments are recorded at once and reversed on overlapping warp tiles.  Where the device has
+ * no memory for that, the segment-wise modes below run, until the record budget is set again.
  * Pipelined, otherwise: a record-mode launch with the full
  * layout and two sweep buffers whose rods each find two free SMs (2 x rods <= SMs) runs
  * every rod on a cluster of two blocks: the first block records the checkpoint segments

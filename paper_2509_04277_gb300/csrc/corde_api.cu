@@ -7,6 +7,7 @@
 #include <climits>
 #include <chrono>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -258,6 +259,7 @@ struct corde_rods {
   float4* d_sweep_rec = nullptr;  // record mode of the reverse pass: sweeps and neighbour data
   size_t sweep_rec_cap = 0;
   long long adj_record_budget = 1ll << 30;
+  size_t adj_tile_limit = SIZE_MAX;  // smallest whole-rollout scratch (float4) that could not be allocated
   int ro_steps = 0, ro_every = 0;
   // last rod_adjoint's largest launch: mode, nt, blocks/SM, blocks, SMs, compact records,
   // pipelined
@@ -785,9 +787,19 @@ int ensure_capacity(float4** buf, size_t* cap, size_t need) {
   cudaFree(*buf);
   *buf = nullptr;
   *cap = 0;
-  CK(cudaMalloc(buf, need * sizeof(float4)));
+  const cudaError_t e = cudaMalloc(buf, need * sizeof(float4));
+  if (e != cudaSuccess) {
+    *buf = nullptr;
+    cudaGetLastError();  // (a later launch must not find it)
+    CK(e);
+  }
   *cap = need;
   return CORDE_OK;
+}
+void release(float4** buf, size_t* cap) {
+  cudaFree(*buf);
+  *buf = nullptr;
+  *cap = 0;
 }
 
 template <class T>
@@ -1303,6 +1315,7 @@ int rod_set_adjoint_record_budget(rod_handle h, long long bytes) {
   if (int rc = check_handle(h)) return rc;
   if (bytes < 0) return fail(CORDE_ERR_ARG, "rod_set_adjoint_record_budget: bytes must be >= 0");
   h->adj_record_budget = bytes;
+  h->adj_tile_limit = SIZE_MAX;
   return CORDE_OK;
 }
 
@@ -1946,7 +1959,9 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
   std::vector<char> compact(h->adj_bins.size(), 0);
   std::vector<char> pipe(h->adj_bins.size(), 0);
   // Tiles: the rods of a bin spread over SMs of their own (one warp per SM partition), when the
-  // records and states of every step fit the budget and the iterations the tiles' ghosts
+  // records and states of every step fit the budget and the iterations the tiles' ghosts.  That is the whole
+  // rollout's scratch, so it is allocated here; without the memory for it the other modes run, whose scratch
+  // is a few segments'.
   std::vector<int> tile_blocks(h->adj_bins.size(), 0);
   size_t sweep_need = 0, seg_need = 0;
   int spare = sms - h->n_rods;
@@ -1956,12 +1971,24 @@ int rod_adjoint(rod_handle h, const float* dL_dpos_traj, float* dL_dK, float* dL
     const size_t rec = (size_t)h->ro_steps * b.count * 2 * iters * 3 * adjoint_tile_npad(b.n_max) / 4;  // float4
     const size_t states = (size_t)(h->ro_steps + 1) * 4 * E;
     if (spare < 0 || (blocks - 1) * b.count > spare ||
-        (long long)((rec + states) * sizeof(float4)) > h->adj_record_budget)
+        (long long)((rec + states) * sizeof(float4)) > h->adj_record_budget || rec + states >= h->adj_tile_limit)
       continue;
     spare -= (blocks - 1) * b.count;
     tile_blocks[i] = blocks;
     sweep_need = std::max(sweep_need, rec);
     seg_need = states;
+  }
+  if (seg_need > 0) {
+    int rc = ensure_capacity(&h->d_seg, &h->seg_cap, seg_need);
+    if (rc == CORDE_OK && sweep_need > 0) rc = ensure_capacity(&h->d_sweep_rec, &h->sweep_rec_cap, sweep_need);
+    if (rc != CORDE_OK && rc != CORDE_ERR_OOM) return rc;
+    if (rc == CORDE_ERR_OOM) {
+      release(&h->d_seg, &h->seg_cap);
+      release(&h->d_sweep_rec, &h->sweep_rec_cap);
+      h->adj_tile_limit = seg_need + sweep_need;  // (not tried again until the budget is set)
+      std::fill(tile_blocks.begin(), tile_blocks.end(), 0);
+      sweep_need = seg_need = 0;
+    }
   }
   for (size_t i = 0; i < h->adj_bins.size(); ++i) {
     if (tile_blocks[i]) continue;

@@ -109,3 +109,43 @@ def test_scratch_that_held_other_values(corde):
     for k in got:
         np.testing.assert_array_equal(got[k], want[k], err_msg=k)
     b.close()
+
+
+def test_without_memory_for_the_whole_rollout(corde):
+    """8 rods of 512 nodes over 700 steps: 0.9 GB of states and records, within the default budget but beyond
+    what the device has left.  The segment-wise modes run instead, with the same gradients."""
+    import torch
+
+    rods = [W.adjoint_rod(512, seed=k) for k in range(8)]
+    a, b = corde.RodBatch(rods), corde.RodBatch(rods)
+    g = None
+    for h in (a, b):
+        traj = h.rollout(700, 20)
+        if g is None:
+            g = torch.zeros_like(traj)
+            g[:, :, :3] = 1e-3 * torch.cos(traj[:, :, :3] * 23.0)
+        del traj
+    want = a.adjoint(g)
+    assert corde.rod_adjoint_kernels(a.handle)["tiles"] == 1
+    a.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = []
+    for keep, piece in ((3 << 30, None), (600 << 20, 256 << 20)):
+        while torch.cuda.mem_get_info()[0] > keep + (piece or 0):
+            hold.append(torch.empty(piece or torch.cuda.mem_get_info()[0] - keep, dtype=torch.uint8, device="cuda"))
+    assert torch.cuda.mem_get_info()[0] < 900 << 20
+    for _ in range(2):
+        got = b.adjoint(g)
+        ran = corde.rod_adjoint_kernels(b.handle)
+        assert ran["tiles"] == 0 and sum(ran.values()) == 1, ran
+        for k in want:
+            assert torch.equal(got[k], want[k]), k
+    hold.clear()
+    torch.cuda.empty_cache()
+    b.set_adjoint_record_budget(1 << 30)
+    got = b.adjoint(g)
+    assert corde.rod_adjoint_kernels(b.handle)["tiles"] == 1
+    for k in want:
+        assert torch.equal(got[k], want[k]), k
+    b.close()
