@@ -577,6 +577,13 @@ int check_handle(rod_handle h) {
   return CORDE_OK;
 }
 
+// Copies bytes from pageable host memory and waits for them: cudaMemcpy may return before they have arrived,
+// and a launch on a stream that does not wait for the legacy one could read what was there before.
+cudaError_t to_device(void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamLegacy);
+}
+
 void free_bins(rod_handle h) {
   for (auto* list : {&h->bins, &h->graph_bins}) {
     for (auto& b : *list) {
@@ -662,7 +669,7 @@ int alloc_bins(rod_handle h) {
     for (const Bin& b : *list) work.insert(work.end(), b.rods.begin(), b.rods.end());
   if (work.empty()) return CORDE_OK;
   CK(cudaMalloc(&h->d_work, work.size() * sizeof(int)));
-  CK(cudaMemcpy(h->d_work, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice));
+  CK(to_device(h->d_work, work.data(), work.size() * sizeof(int)));
   int* d = h->d_work;
   for (auto* list : {&h->bins, &h->graph_bins})
     for (Bin& b : *list) {
@@ -672,14 +679,13 @@ int alloc_bins(rod_handle h) {
         const size_t n4 = (size_t)b.count * 2 * b.cluster * 2 * kHaloSlots;
         CK(cudaMalloc(&b.d_gh, n4 * sizeof(float4)));
         CK(cudaMemset(b.d_gh, 0, n4 * sizeof(float4)));
+        CK(cudaStreamSynchronize(cudaStreamLegacy));
       }
       if (b.tile.per && b.tile.grid) {
         const int64_t bytes = tile_halo_bytes(b.tile.per, b.n_max);
         CK(cudaMalloc(&b.d_tile_gh, bytes));
         CK(cudaMemset(b.d_tile_gh, 0, bytes));  // no stamps
-        CK(cudaMemcpy(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &h->wait_limit, sizeof(unsigned),
-                      cudaMemcpyHostToDevice));
-        CK(cudaStreamSynchronize(cudaStreamLegacy));  // before a launch on a stream that doesn't wait for this one
+        CK(to_device(tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 2, &h->wait_limit, sizeof(unsigned)));
       }
     }
   return CORDE_OK;
@@ -1492,10 +1498,11 @@ int rod_autotune(rod_handle h, int n_steps, void* stream) {
         mine.push_back(b);
       }
       h->plan = kept;
-      cudaMemcpy(d_work, work.data(), work.size() * sizeof(int), cudaMemcpyHostToDevice);
+      if (to_device(d_work, work.data(), work.size() * sizeof(int)) != cudaSuccess) mine.clear();
       return mine;
     };
     auto run = [&](const std::vector<Bin>& bins) {
+      if (bins.empty()) return fail(CORDE_ERR_CUDA, "autotune work list");
       if (bins.size() == 1) return launch_bins(h, bins.data(), 1, n_steps, h->d_drive, s);
       if (int e = prepare_fork(h, bins.size())) return e;
       cudaError_t e = cudaSuccess;
@@ -1725,7 +1732,7 @@ static int build_pair_bins(rod_handle h) {
         }
       }
       CK(cudaMalloc(&pb.d_pairs, ps.size() * sizeof(int4)));
-      CK(cudaMemcpy(pb.d_pairs, ps.data(), ps.size() * sizeof(int4), cudaMemcpyHostToDevice));
+      CK(to_device(pb.d_pairs, ps.data(), ps.size() * sizeof(int4)));
       h->pair_bins.push_back(pb);
     }
   return CORDE_OK;
@@ -1848,7 +1855,7 @@ static int build_adjoint_bins(rod_handle h) {
     if (v < 0) return fail(CORDE_ERR_UNSUPPORTED, "no <2, " + std::to_string(nt) + "> step variant");
     Bin b{v, (int)rods.size(), nullptr};
     CK(cudaMalloc(&b.d_work, rods.size() * sizeof(int)));
-    CK(cudaMemcpy(b.d_work, rods.data(), rods.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CK(to_device(b.d_work, rods.data(), rods.size() * sizeof(int)));
     for (int r : rods) b.n_max = std::max(b.n_max, h->n_nodes[r]);
     if (h->tiles) b.tile = tile_plan(b.n_max, b.count, 2, &room);
     // two or more tiles in one block don't pay here: a training step of 256 rods of 256 nodes took
