@@ -220,8 +220,9 @@ int rod_diagnostics(rod_handle h, double* out);
  * A plan fixes the arithmetic: the order in which an element's contributions are added and
  * the form of the impulses follow from ept.  Without a mailbox, rods that leave SMs idle run
  * as overlapping warp tiles over several of them, and rods of one tile as one warp, with the
- * results of the plan bit for bit; rod_get_plan still reports the plan.  Tiles of a long rod
- * meet at cluster or grid barriers of blocks that are resident together. */
+ * results of the plan bit for bit; rod_get_plan still reports the plan, rod_get_kernels what
+ * runs.  Tiles of a long rod meet at cluster barriers, or on a grid wait for their neighbours'
+ * data; their blocks are resident together. */
 int rod_set_plan(rod_handle h, int ept, int nt);
 
 /* Warp tiles (on by default): enable = 0 keeps every rod, pair and reverse pass on the block,
@@ -255,7 +256,8 @@ int rod_get_kernels(rod_handle h, int* out);
 /* Launch overlap (on by default): the stepping kernels are launched with programmatic
  * stream serialisation, so a launch is scheduled while the stream's previous stepping
  * kernel still runs and starts stepping as soon as that kernel's writes are visible (each
- * kernel waits for them before its first global access).  Results are bit for bit those
+ * kernel waits for them before it reads or writes state, drive or joint parameters).  Results
+ * are bit for bit those
  * of ordinary launches; enable = 0 switches it off (e.g. to time the launch gap).
  * enable must be 0 or 1 (CORDE_ERR_ARG otherwise).  Host-side only. */
 int rod_set_launch_overlap(rod_handle h, int enable);
@@ -263,8 +265,10 @@ int rod_set_plan_cluster(rod_handle h, int ept, int nt, int cluster);
 /* A rod longer than a 16-block cluster holds (32768 nodes) runs on a cooperative grid
  * of `blocks` blocks (the paper's multi-block kernel, Section 2.2, over the whole GPU):
  * each block's first and last thread publish their exchange slots in global memory and
- * every exchange barrier is a grid sync; the runtime launches the grid only when all its
- * blocks are resident at once, so a sync never waits on a block that is not running.
+ * every exchange barrier of the grid kernel is a grid sync; a lone rod's tiles wait for their
+ * neighbours' data instead, with a limit (rod_set_wait_limit), and beyond eight warps per SM at
+ * one grid sync a step.  The runtime launches the grid only when all its blocks are
+ * resident at once, so neither waits on a block that is not running.
  * rod_create gives such a rod 2048 nodes per block (ept 4, nt 512); the longest rod is
  * 2048 x the blocks the device holds at once (one per SM at nt 512).
  * rod_set_plan_grid forces the grid form of a cluster variant (ept, nt) in {(2,256),

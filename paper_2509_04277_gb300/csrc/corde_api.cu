@@ -127,8 +127,8 @@ int default_variant(int n) {
   return best;
 }
 
-// The block of `threads` threads (a multiple of 32) with four elements per thread, NULL if the
-// variants themselves are the smallest that hold it.
+// The block of `threads` threads with four elements per thread that is no plan of its own (multiples of 32
+// between the powers of two), NULL for other counts.
 const StepVariant* trimmed_variant(int threads) {
   const std::pair<const StepVariant*, int> t[] = {
       {kStepTrimA, kNumStepTrimA}, {kStepTrimB, kNumStepTrimB}, {kStepTrimC, kNumStepTrimC}};
@@ -614,8 +614,9 @@ TileRoom tile_room(rod_handle h) {
 // The handle's rods in bins of one launch each: by plan, and with by_trim also by the smallest block
 // that holds them.  Nothing is allocated here.
 std::vector<Bin> list_bins(rod_handle h, bool by_trim) {
-  // Threads of the block, in steps of 32 between the powers of two, that a rod's <4, *> variant can shrink
-  // to; 0: none is smaller.  Power-of-two blocks are on average 28 % idle warps for log-uniform lengths,
+  // Threads of the smallest block that holds the rod, where that is smaller than its <4, *> variant's and no
+  // power of two; 0: the variant's own block runs (also where a smaller power of two would hold the rod: the
+  // plan is then the caller's or the tuner's choice).  Power-of-two blocks are on average 28 % idle warps for log-uniform lengths,
   // which take issue slots in the constraint sweeps and keep other blocks off the SM.
   auto trim_of = [&](int r, int n) {
     if (h->plan_cluster[r] != 0 || variants()[h->plan[r]].ept != 4) return 0;

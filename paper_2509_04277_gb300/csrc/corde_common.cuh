@@ -94,9 +94,10 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // Programmatic dependent launch.  A stepping kernel starts with this: it lets the stream's
 // next kernel be scheduled at once (that kernel only starts its own prologue early), then
 // waits until the stream's previous kernel has completed and its writes are visible.  Every
-// global access of the kernel comes after the wait, so the result does not depend on
-// whether the launch carried the programmatic-serialisation attribute (without it the wait
-// returns at once).
+// access to what a kernel may have written comes after the wait, so the result does not
+// depend on whether the launch carried the programmatic-serialisation attribute (without it
+// the wait returns at once).  Only the work list, the pairs and the rod constants may be read
+// before it (the tile kernels do): the host writes them, and waits until they have arrived.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

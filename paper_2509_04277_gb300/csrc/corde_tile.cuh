@@ -365,6 +365,11 @@ struct TileLink {
   // the barrier of an exchange: it orders the tiles' shared-memory buffers (global memory on a grid of many warps)
   // and nothing else.  The full cluster barrier also waits for a block's global accesses in
   // flight, the adjoint's prefetches above all.
+  // A tile's reads of a neighbour's buffer are not ordered by it: the release is that of the block's own shared
+  // memory, and the arrive is relaxed.  They are complete all the same, since whatever a ghost lane reads in one
+  // exchange goes into the step's arithmetic (forces, sweeps, positions, the reverse step), whose results the
+  // warp stores into its own buffer before the next meet, and the neighbour rewrites the buffer that was read only
+  // after that one.  An exchange of values that are not used before the next one would need a full barrier.
   __device__ __forceinline__ void meet() const {
     if constexpr (SYNC == kTileCluster) {
       asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
@@ -401,7 +406,10 @@ struct TileLink {
   }
   // On a grid a tile waits for its two neighbours only, by polling the data itself.  A tile
   // publishes exchange i only after it has read its neighbours' exchange i - 1, and they published
-  // that after they had read its exchange i - 2: two buffers suffice.
+  // that after they had read its exchange i - 2: two buffers suffice.  Nothing else orders these accesses:
+  // they are relaxed, and the vote orders no memory.  Within a warp the reads come first because the vote needs
+  // every lane's stamps (a slot's stamp and floats are one access); between warps a slot read too late
+  // would carry a newer stamp, which the loop does not take.
   template <int N>
   __device__ __forceinline__ bool trade_stamped(float4 (&a)[N]) {
     constexpr int M = (4 * N + 2) / 3;
