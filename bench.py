@@ -118,7 +118,7 @@ class ClockSampler:
 
 def _kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("corde_step.cuh", "corde_common.cuh"):
+    for f in ("corde_step.cuh", "corde_common.cuh", "corde_tile.cuh", "corde_tile.cu"):
         with open(os.path.join(ROOT, "paper_2509_04277_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -828,7 +828,7 @@ def main_ours(args):
         n_sms = fp32["n_sms"]
         flops_launch = flops_per_el_step(single["n_iters"]) * single["n_nodes"] * STEPS_PER_LAUNCH
         achieved = flops_launch / (single["kernel_ms_avg"] * 1e-3) / 1e12
-        traffic, _ = _traffic("step_kernel_guidewire512")
+        traffic, _ = _traffic("tile_step_kernel_guidewire512")
         cpu = cpu_baseline_single(args.cpu_seconds)
         out = {
             "metric": METRIC,
