@@ -267,7 +267,9 @@ int rod_set_plan_cluster(rod_handle h, int ept, int nt, int cluster);
  * each block's first and last thread publish their exchange slots in global memory and
  * every exchange barrier of the grid kernel is a grid sync; a lone rod's tiles wait for their
  * neighbours' data instead, with a limit (rod_set_wait_limit), and beyond eight warps per SM at
- * one grid sync a step.  The runtime launches the grid only when all its blocks are
+ * one grid sync a step.  Those tiles take most SMs (rod_get_kernels): beside other handles'
+ * launches that hold SMs for long, rod_set_tiles(h, 0) keeps the rod on its plan's blocks.
+ * The runtime launches the grid only when all its blocks are
  * resident at once, so neither waits on a block that is not running.
  * rod_create gives such a rod 2048 nodes per block (ept 4, nt 512); the longest rod is
  * 2048 x the blocks the device holds at once (one per SM at nt 512).

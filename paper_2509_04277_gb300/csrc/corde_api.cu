@@ -188,11 +188,14 @@ TilePlan tile_plan(int n, int count, int arith, TileRoom* room) {
   const int K = p.per == 2 ? K2 : K4;
   p.blocks = std::min((K + 3) / 4, kMaxCluster);
   if (K > 8 * p.blocks) {
-    // more tiles than a cluster holds: a cooperative grid, one block per SM
+    // more tiles than a cluster holds: a cooperative grid, one block per SM.  Such a grid starts only when all
+    // its blocks find SMs, so it takes no more of them than the warps per block need (65536 nodes: 137 blocks
+    // of six warps): another handle's running launch (a mailbox) can hold the others meanwhile.
     p.grid = 1;
     p.blocks = std::min(K, room->spare + 1);
   }
   p.warps = p.blocks > 0 ? (K + p.blocks - 1) / p.blocks : 0;
+  if (p.grid && p.warps > 0) p.blocks = (K + p.warps - 1) / p.warps;
   p.full = p.grid && p.warps > kTileMaxWarps;  // up to 16 warps on every SM
   const int64_t more = (int64_t)(p.blocks - 1) * count;
   if (p.blocks >= 1 && p.warps <= (p.full ? 2 : 1) * kTileMaxWarps && !(p.grid && count > 1) && room->spare >= more) {

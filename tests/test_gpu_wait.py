@@ -64,3 +64,36 @@ def test_nothing_lost_without_a_cause(corde):
     b.step(50)
     assert corde.rod_wait_status(b.handle) == 0
     b.close()
+
+
+@pytest.mark.parametrize("n", [20000, 65536])
+def test_grid_beside_a_running_launch(corde, n):
+    """A lock-step launch of another handle holds its SM until its wait for the host runs out, after 1 s; the
+    grid's steps start and end meanwhile."""
+    import time
+
+    import torch
+
+    a, b, c = corde.RodBatch([W.guidewire(512, seed=1)]), corde.RodBatch([W.guidewire(n, seed=2)]), corde.RodBatch([W.guidewire(n, seed=2)])
+    c.step(10)
+    c.step(10)
+    want = c.state_numpy()
+    a.step(10)
+    corde.rod_mailbox_enable(a.handle, 10, 64)
+    corde.rod_mailbox_lockstep(a.handle, True, 1_000_000)
+    sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    t0 = time.time()
+    a.step(50, stream=sa)
+    for _ in range(2):
+        b.step(10, stream=sb)
+    sb.synchronize()
+    took = time.time() - t0
+    sa.synchronize()
+    assert corde.rod_mailbox_status(a.handle) & 1  # it did run, and waited
+    assert took < 0.5 <= time.time() - t0
+    st = b.state_numpy()
+    for k in want:
+        np.testing.assert_array_equal(st[k].view(np.uint32), want[k].view(np.uint32), err_msg=k)
+    for h in (a, b, c):
+        h.close()
