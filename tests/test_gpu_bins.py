@@ -58,7 +58,7 @@ def test_lockstep_rods_of_one_plan_run_together(corde):
     b.close()
 
 
-@pytest.mark.parametrize("lengths", [LENGTHS, (300, 600, 900, 40)])
+@pytest.mark.parametrize("lengths", [LENGTHS, (300, 600, 900, 40), (12000, 300, 5000)])
 def test_caller_capture(corde, lengths):
     """A step in a caller's capture, the first of its handle or a repeated one, replays like direct steps."""
     import torch
