@@ -619,8 +619,8 @@ TileRoom tile_room(rod_handle h) {
 std::vector<Bin> list_bins(rod_handle h, bool by_trim) {
   // Threads of the smallest block that holds the rod, where that is smaller than its <4, *> variant's and no
   // power of two; 0: the variant's own block runs (also where a smaller power of two would hold the rod: the
-  // plan is then the caller's or the tuner's choice).  Power-of-two blocks are on average 28 % idle warps for log-uniform lengths,
-  // which take issue slots in the constraint sweeps and keep other blocks off the SM.
+  // plan is then the caller's or the tuner's choice).  Power-of-two blocks are on average 28 % idle warps
+  // for log-uniform lengths, which take issue slots in the constraint sweeps and keep other blocks off the SM.
   auto trim_of = [&](int r, int n) {
     if (h->plan_cluster[r] != 0 || variants()[h->plan[r]].ept != 4) return 0;
     const int t = ((n + 3) / 4 + 31) / 32 * 32;
@@ -898,7 +898,7 @@ int launch_forked(rod_handle h, const std::vector<Bin>& bins, int n_steps, const
   *e = cudaEventRecord(h->fork_ev, s);
   for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) *e = cudaStreamWaitEvent(h->side[k], h->fork_ev, 0);
   const int pdl = h->pdl;
-  if (s != h->cap_stream) h->pdl = 0;  // (a branch starts with an event wait: there is no kernel to overlap with)
+  if (!h->cap_stream || s != h->cap_stream) h->pdl = 0;  // (a branch starts with an event wait: there is no kernel to overlap with)
   if (*e == cudaSuccess) rc = launch_all(h, bins, n_steps, d, s, &h->side, nullptr, pairs);
   h->pdl = pdl;
   for (size_t k = 0; k < nb && *e == cudaSuccess; ++k) {
@@ -1794,15 +1794,16 @@ int rod_wait_status(rod_handle h, int* n_lost) {
   if (!n_lost) return fail(CORDE_ERR_ARG, "rod_wait_status: NULL argument");
   CK(cudaDeviceSynchronize());
   *n_lost = 0;
-  for (auto* list : {&h->bins, &h->graph_bins}) for (const Bin& b : *list) {
-    if (!b.d_tile_gh) continue;
-    unsigned* word = tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 1;
-    unsigned lost = 0;
-    CK(cudaMemcpy(&lost, word, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    if (lost == 0) continue;
-    ++*n_lost;
-    CK(cudaMemset(word, 0, sizeof(unsigned)));
-  }
+  for (auto* list : {&h->bins, &h->graph_bins})
+    for (const Bin& b : *list) {
+      if (!b.d_tile_gh) continue;
+      unsigned* word = tile_tail(b.d_tile_gh, b.tile.per, b.n_max) + 1;
+      unsigned lost = 0;
+      CK(cudaMemcpy(&lost, word, sizeof(unsigned), cudaMemcpyDeviceToHost));
+      if (lost == 0) continue;
+      ++*n_lost;
+      CK(cudaMemset(word, 0, sizeof(unsigned)));
+    }
   CK(cudaDeviceSynchronize());
   return CORDE_OK;
 }
